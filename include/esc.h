@@ -369,7 +369,7 @@ esc_status esc_selftest_wait_timeout(uint64_t limit_ns, void *stream);
  * esc_debug_write_units(nrows, slots, ...): the compaction units a
  * materialising call on a table of nrows rows (<= ESC_MAX_ROWS) uses when
  * the GPU holds `slots` write-kernel blocks at once (slots = 0: the
- * full-size units of a batch); out (host, 3 entries): the groups of 256
+ * full-size units); out (host, 3 entries): the groups of 256
  * rows per unit, the number of units, and the reciprocal that maps a group
  * to its unit (ceil(2^32 / groups per unit), 0 for one group). */
 esc_status esc_debug_fail_allocs(int32_t n);

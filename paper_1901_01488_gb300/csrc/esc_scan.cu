@@ -1678,6 +1678,17 @@ uint32_t tile_rows_for(const Query &q, const esc_tuning &tu) {
   return std::min<uint32_t>(std::min<uint32_t>(t, kMaxTileRows), tu.max_tile_rows);
 }
 
+// Splits a query's groups into compaction units of `ug` groups (1..kMaxUnitGroups).
+void set_write_units(Query &q, uint64_t ug) {
+  const uint64_t ngroups = ((uint64_t)q.nrows + kGroup - 1) / kGroup;
+  q.wunit_groups = (uint32_t)ug;
+  // group g's unit is g / ug = umulhi(g, ceil(2^32 / ug)): with ug * M = 2^32 + e,
+  // e < ug, the quotient is exact while g * e < 2^32, and every group index
+  // (< ESC_MAX_ROWS / 256 < 2^24) keeps g * 255 below 2^32
+  q.wunit_recip = ug > 1 ? (uint32_t)(((1ull << 32) + ug - 1) / ug) : 0u;
+  q.nwunits = (uint32_t)((ngroups + ug - 1) / ug);
+}
+
 // Compaction units: one write-kernel block each.  slots == 0: units of
 // kMaxUnitGroups groups.  Otherwise the fewest whole waves of `slots` blocks
 // that full-size units need, with units just large enough to fill them: the
@@ -1691,12 +1702,29 @@ void layout_write_units(Query &q, int slots) {
     const uint64_t waves = std::max<uint64_t>(1, (ngroups + wave - 1) / wave);
     ug = std::min<uint64_t>(kMaxUnitGroups, std::max<uint64_t>(1, (ngroups + waves * slots - 1) / (waves * slots)));
   }
-  q.wunit_groups = (uint32_t)ug;
-  // group g's unit is g / ug = umulhi(g, ceil(2^32 / ug)): with ug * M = 2^32 + e,
-  // e < ug, the quotient is exact while g * e < 2^32, and every group index
-  // (< ESC_MAX_ROWS / 256 < 2^24) keeps g * 255 below 2^32
-  q.wunit_recip = ug > 1 ? (uint32_t)(((1ull << 32) + ug - 1) / ug) : 0u;
-  q.nwunits = (uint32_t)((ngroups + ug - 1) / ug);
+  set_write_units(q, ug);
+}
+
+// Compaction units of the sub-queries that share one write launch (a batch
+// or one of its waves): one unit size for all of them, such that the launch
+// has about kBatchWriteWaves waves of resident blocks, 8 to kMaxUnitGroups
+// groups a unit.  A block's time follows its unit's qualifying rows, so large
+// units leave the few dense ones as the launch's tail: with 256-group units
+// the early waves of a 96-query batch ran 16 to 55 blocks on 152 SMs, 75 to
+// 121 us each.  Measured, that batch (10K to 8M rows, 10 waves): 1972 us with
+// 256-group units, 1581 / 1545 / 1536 / 1667 us at 1 / 2 / 4 / 8 waves of
+// blocks; the smallest unit (4, 8 or 16 groups) moves it by under 1 %.
+constexpr int kBatchWriteWaves = 2;
+constexpr uint64_t kMinBatchUnitGroups = 8;
+void layout_batch_write_units(Query *qs, int n, int sms) {
+  uint64_t groups = 0;
+  for (int i = 0; i < n; ++i)
+    if (qs[i].mode == MODE_SELECT && !qs[i].is_const) groups += ((uint64_t)qs[i].nrows + kGroup - 1) / kGroup;
+  const uint64_t blocks = (uint64_t)kBatchWriteWaves * sms * kWriteBlocksPerSm;
+  const uint64_t ug =
+      std::min<uint64_t>(kMaxUnitGroups, std::max<uint64_t>(kMinBatchUnitGroups, (groups + blocks - 1) / blocks));
+  for (int i = 0; i < n; ++i)
+    if (qs[i].mode == MODE_SELECT && !qs[i].is_const) set_write_units(qs[i], ug);
 }
 
 // Stage layout (read columns back to back, each slice 128-byte aligned), the
@@ -1995,7 +2023,6 @@ esc_status batch_prepare(const esc_table *const *tables, const esc_pred *const *
     if ((s = prepare_query(tables[i], preds[i], compact ? r : nullptr, compact ? MODE_SELECT : MODE_COUNT,
                            &qin[i])) != ESC_OK)
       return s;
-    layout_write_units(qin[i], 0);  // one write grid for all queries: full-size units
     mark_constant(qin[i]);
   }
   // smallest work first (stable: equal work keeps the caller's order)
@@ -2027,6 +2054,7 @@ esc_status batch_prepare(const esc_table *const *tables, const esc_pred *const *
   uint64_t zeroed = 0, other = 0;
   for (int w = 0, k0 = 0; w < nw; k0 = wend[w++]) {
     uint64_t units = 0, wunits = 0;
+    layout_batch_write_units(&qs[k0], wend[w] - k0, d->sms);  // one write grid per wave
     for (int k = k0; k < wend[w]; ++k) {
       Query &q = qs[k];
       if (q.is_const) cidx.push_back((uint32_t)k);
@@ -2229,8 +2257,13 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
     if ((s = prepare_query(tables[i], preds[i], compact ? r : nullptr, compact ? MODE_SELECT : MODE_COUNT,
                            &qs[i])) != ESC_OK)
       return s;
-    layout_write_units(qs[i], 0);  // one write grid for all queries: full-size units
     mark_constant(qs[i]);
+  }
+  DeviceState *d;
+  if ((s = device_state(&d)) != ESC_OK) return s;
+  layout_batch_write_units(qs.data(), n, d->sms);  // one write grid for all queries
+  for (int i = 0; i < n; ++i) {
+    const bool compact = qs[i].mode == MODE_SELECT;
     if (qs[i].is_const) cidx.push_back((uint32_t)i);
     qs[i].unit_base = (uint32_t)units;
     qs[i].wunit_base = (uint32_t)wunits;

@@ -389,7 +389,7 @@ def esc_debug_fail_allocs(n: int) -> None:
 def esc_debug_write_units(nrows: int, slots: int) -> Tuple[int, int, int]:
     """(groups per compaction unit, units, group-to-unit reciprocal) of a
     materialising call on `nrows` rows with `slots` write-kernel blocks
-    resident (0: a batch's full-size units)."""
+    resident (0: full-size units)."""
     out = (ctypes.c_uint32 * 3)()
     _check(_lib.esc_debug_write_units(nrows, slots, out), "esc_debug_write_units")
     return out[0], out[1], out[2]

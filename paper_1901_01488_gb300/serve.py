@@ -73,9 +73,9 @@ def request_bytes(nrows: int, req: Request, widths: Dict[str, int]) -> int:
     counters in the launch (4 KB), and when it materialises, the library's
     scratch (the selection bitmap, 1/8 byte per row rounded up to whole tiles
     of at most 32768 rows; 16 bytes per compaction unit, of which there are
-    at most one per 256-row group and at most one per 65536 rows plus one
-    wave of write-kernel blocks, taken as 1024; headers) and its output
-    buffers."""
+    at most one per 256-row group and at most one per 65536 rows plus two
+    waves of write-kernel blocks, taken as 1024 here and the rest within the
+    8 KB of headers) and its output buffers."""
     base = 4096
     if not req.proj:
         return base
