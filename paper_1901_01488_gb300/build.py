@@ -22,9 +22,10 @@ LIB = os.path.join(HERE, "libesc.so")
 LIB_CHECKED = os.path.join(HERE, "libesc_checked.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU = ["esc_scan.cu", "esc_semijoin.cu", "esc_mlp.cu"]
-CPP = ["esc_host.cpp"]
-HEADERS = [os.path.join(CSRC, "esc_internal.h"), os.path.join(ROOT, "include", "esc.h")]
+CU = ["esc_scan.cu", "esc_boxes.cu", "esc_semijoin.cu", "esc_mlp.cu"]
+CPP = ["esc_host.cpp", "esc_stage.cpp"]
+HEADERS = [os.path.join(CSRC, h) for h in ("esc_internal.h", "esc_boxes.h", "esc_ptx.cuh", "esc_stage.h")] + [
+    os.path.join(ROOT, "include", "esc.h")]
 
 
 def _stale(target: str, deps) -> bool:

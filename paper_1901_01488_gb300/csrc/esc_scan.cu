@@ -32,11 +32,15 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
+#include "esc_boxes.h"
 #include "esc_internal.h"
+#include "esc_ptx.cuh"
 
 namespace esc {
 
@@ -50,109 +54,7 @@ constexpr int kStages = 3;
 constexpr uint32_t kStageBytes = 64 * 1024;
 constexpr int kTailTilesPerSm = 8;      // single-tile work units at the end of a query (per SM)
 constexpr int kMaxUnitGroups = kMaxUnitRows / kGroup;  // 256: one write-kernel thread per group
-constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s per bounded wait
-constexpr uint32_t FULL = 0xffffffffu;
 static_assert(kStageBytes <= 65536, "stage column offsets are 16-bit");
-
-// ------------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(bar))
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
-                   smem_addr(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(bar))
-      : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t lanemask_lt() {
-  uint32_t m;
-  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-  return m;
-}
-
-__device__ __forceinline__ void raise_status(ScratchHdr *hdr, unsigned status) {
-  atomicCAS(&hdr->status, 0u, status);
-  atomicExch(&hdr->abort, 1u);
-}
-__device__ __forceinline__ bool aborted(const ScratchHdr *hdr) {
-  return *(volatile const unsigned *)&hdr->abort != 0u;
-}
-
-// Warp-collective bounded wait for the phase of parity `parity` of an
-// mbarrier: every lane must observe the completion itself (so that every lane
-// has acquire ordering), the warp leaves together, and the decision to give
-// up is lane 0's, broadcast.  With `abortable` the wait also gives up as
-// soon as the launch is aborting (used for every wait that does not guard an
-// in-flight bulk copy, so that one timeout cannot cascade into more).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, ScratchHdr *hdr,
-                                          uint64_t limit_ns = kWaitLimitNs, bool abortable = false) {
-  bool seen = mbar_try_wait(bar, parity);
-  if (__all_sync(FULL, seen)) return true;
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    if (!seen) seen = mbar_try_wait(bar, parity);
-    if (__all_sync(FULL, seen)) return true;
-    if ((it & 63u) == 0) {
-      int give_up = 0;
-      if ((threadIdx.x & 31) == 0) give_up = (abortable && aborted(hdr)) ? 1 : (globaltimer() - t0 > limit_ns) ? 2 : 0;
-      give_up = __shfl_sync(FULL, give_up, 0);
-      if (give_up) {
-        if (give_up == 2 && (threadIdx.x & 31) == 0) raise_status(hdr, ESC_ETIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
-// Warp-collective non-blocking test: true only if every lane observed it.
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return __all_sync(FULL, ok != 0);
-}
 
 // ------------------------------------------------------------------ loads
 // Values of this lane's 8 rows of a group, for each element type (see the
@@ -2338,60 +2240,109 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
   return s;
 }
 
+// Whether n predicates over `rows` rows are counted by table lookup.  It costs
+// two launches more (about 25 us) and the rows' intervals, whatever n;
+// interpreting costs about 2.3 us per predicate and million rows, and from 17
+// predicates on about 1 us per predicate to copy their programs.  Both
+// measured, lookup / interpreter, us: 8M rows: 4 predicates 111 / 80, 8 154 /
+// 148, 12 162 / 239, 16 138 / 302, 32 195 / 554; 1M: 8 61 / 38, 12 58 / 53, 16
+// 54 / 64, 32 73 / 115; 100K: 16 46 / 37, 32 53 / 66; 10K: 32 52 / 54, 64 59 / 92.
+inline bool lookup_pays(int32_t n, uint64_t rows) { return n >= 12 && (n >= 32 || rows * (uint64_t)n >= 16000000u); }
+
 // One shared scan: `n` count-only predicates of table t whose read columns
-// (union `ucols`, table column indices) fit one stage layout.
+// (union `ucols`, table column indices) fit one stage layout.  Predicates that
+// decompose into boxes are counted by table lookup (esc_boxes.cu), in as many
+// passes as their limits ask for; the others are interpreted.
 static esc_status run_shared_group(const esc_table *t, const esc_pred *const *preds, int32_t n,
                                    const std::vector<int32_t> &ucols, uint64_t *dev_counts, cudaStream_t st) {
   DeviceState *d;
   esc_status s = device_state(&d);
   if (s != ESC_OK) return s;
-  Launch L;
-  std::memset(&L, 0, sizeof L);
-  Query &Y = L.q0;
-  Y.nrows = (uint32_t)t->nrows;
-  Y.mode = MODE_COUNT;
-  Y.nref = (int32_t)ucols.size();
-  for (size_t k = 0; k < ucols.size(); ++k) {
-    Y.ref_w[k] = (uint8_t)dtype_width(t->dtypes[ucols[k]]);
-    Y.ref_ptr[k] = static_cast<const uint8_t *>(t->data[ucols[k]]);
-  }
-  layout_stage(Y, d->sms, kDefaultTuning);
-  std::vector<Query> qs((size_t)n);
-  for (int k = 0; k < n; ++k) {
-    if ((s = prepare_query(t, preds[k], nullptr, MODE_COUNT, &qs[k])) != ESC_OK) return s;
-    auto uslot = [&](int local) {
-      const int32_t col = preds[k]->ref_cols[local];
-      return (int)(std::find(ucols.begin(), ucols.end(), col) - ucols.begin());
-    };
-    for (int pc = 0; pc < qs[k].ninstr; ++pc) {  // stage offsets into the union layout
-      Instr &I = qs[k].code[pc];
-      if (I.op == OP_RANGE || I.op == OP_IN || I.op == OP_INSET || I.op == OP_UDF)
-        I.soff = (uint16_t)Y.stage_off[uslot(I.ref)];
-      if (I.op == OP_UDF) I.soff2 = (uint16_t)Y.stage_off[uslot(I.ref2)];
-    }
-  }
   const size_t head = 256;
   const size_t cnt_bytes = ((size_t)n * 8 + 255) & ~(size_t)255;
-  const size_t q_bytes = sizeof(Query) * (size_t)n;
   void *mem = nullptr;
-  if ((s = alloc_async(&mem, head + cnt_bytes + q_bytes, st)) != ESC_OK) return s;
+  if ((s = alloc_async(&mem, head + cnt_bytes + sizeof(Query) * (size_t)n, st)) != ESC_OK) return s;
+  struct Free {
+    void *mem;
+    cudaStream_t st;
+    ~Free() { cudaFreeAsync(mem, st); }
+  } free_mem{mem, st};
   uint8_t *base = static_cast<uint8_t *>(mem);
+  ScratchHdr *hdr = reinterpret_cast<ScratchHdr *>(base);
   unsigned long long *counts = reinterpret_cast<unsigned long long *>(base + head);
   Query *dq = reinterpret_cast<Query *>(base + head + cnt_bytes);
-  for (int k = 0; k < n; ++k) qs[k].count = &counts[k];
   cudaError_t e = cudaMemsetAsync(base, 0, head + cnt_bytes, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dq, qs.data(), q_bytes, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && Y.nunits > 0) {
-    L.queries = dq;
-    L.nq = n;
-    L.total_units = Y.nunits;
-    L.hdr = reinterpret_cast<ScratchHdr *>(base);
-    const uint32_t grid = std::min<uint32_t>((uint32_t)(d->sms * d->blocks_per_sm), Y.nunits);
-    shared_kernel<<<grid, kThreads, SharedSmem::total, st>>>(L);
-    e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_selectivity_shared_async: ") + cudaGetErrorString(e));
+
+  std::vector<int32_t> rest;   // predicates left to the interpreter
+  if (t->nrows > 0 && lookup_pays(n, t->nrows)) {
+    std::unique_ptr<BoxPlan, void (*)(BoxPlan *)> plan(new_box_plan(), free_box_plan);
+    std::vector<int32_t> in;   // the plan's predicates
+    auto flush = [&]() -> esc_status {
+      bool done = in.empty();
+      if (!done) {
+        const esc_status fs = run_boxes(plan.get(), t, d->sms, counts, hdr, st, &done);
+        if (fs != ESC_OK) return fs;
+      }
+      if (!done) rest.insert(rest.end(), in.begin(), in.end());
+      in.clear();
+      plan.reset(new_box_plan());
+      return ESC_OK;
+    };
+    for (int32_t k = 0; k < n; ++k) {
+      BoxFit fit = add_predicate(plan.get(), preds[k], (uint32_t)k);
+      if (fit == BOX_FULL) {
+        if ((s = flush()) != ESC_OK) return s;
+        fit = add_predicate(plan.get(), preds[k], (uint32_t)k);
+      }
+      if (fit == BOX_ADDED) in.push_back(k);
+      else rest.push_back(k);
+    }
+    if ((s = flush()) != ESC_OK) return s;
+  } else if (t->nrows > 0) {
+    for (int32_t k = 0; k < n; ++k) rest.push_back(k);
+  }
+
+  if (!rest.empty()) {
+    Launch L;
+    std::memset(&L, 0, sizeof L);
+    Query &Y = L.q0;
+    Y.nrows = (uint32_t)t->nrows;
+    Y.mode = MODE_COUNT;
+    Y.nref = (int32_t)ucols.size();
+    for (size_t k = 0; k < ucols.size(); ++k) {
+      Y.ref_w[k] = (uint8_t)dtype_width(t->dtypes[ucols[k]]);
+      Y.ref_ptr[k] = static_cast<const uint8_t *>(t->data[ucols[k]]);
+    }
+    layout_stage(Y, d->sms, kDefaultTuning);
+    HostStage stage(sizeof(Query) * rest.size(), st);
+    Query *qs = reinterpret_cast<Query *>(stage.data());
+    for (size_t k = 0; k < rest.size(); ++k) {
+      const esc_pred *p = preds[rest[k]];
+      if ((s = prepare_query(t, p, nullptr, MODE_COUNT, &qs[k])) != ESC_OK) return s;
+      qs[k].count = &counts[rest[k]];
+      auto uslot = [&](int local) {
+        return (int)(std::find(ucols.begin(), ucols.end(), p->ref_cols[local]) - ucols.begin());
+      };
+      for (int pc = 0; pc < qs[k].ninstr; ++pc) {  // stage offsets into the union layout
+        Instr &I = qs[k].code[pc];
+        if (I.op == OP_RANGE || I.op == OP_IN || I.op == OP_INSET || I.op == OP_UDF)
+          I.soff = (uint16_t)Y.stage_off[uslot(I.ref)];
+        if (I.op == OP_UDF) I.soff2 = (uint16_t)Y.stage_off[uslot(I.ref2)];
+      }
+    }
+    e = stage.copy_to(dq);
+    if (e == cudaSuccess) {
+      L.queries = dq;
+      L.nq = (int32_t)rest.size();
+      L.total_units = Y.nunits;
+      L.hdr = hdr;
+      const uint32_t grid = std::min<uint32_t>((uint32_t)(d->sms * d->blocks_per_sm), Y.nunits);
+      shared_kernel<<<grid, kThreads, SharedSmem::total, st>>>(L);
+      e = cudaGetLastError();
+    }
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(dev_counts, counts, (size_t)n * 8, cudaMemcpyDeviceToDevice, st);
-  cudaFreeAsync(mem, st);
   if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_selectivity_shared_async: ") + cudaGetErrorString(e));
   return ESC_OK;
 }
@@ -2406,20 +2357,24 @@ esc_status esc_selectivity_shared_async(const esc_table *t, const esc_pred *cons
       return fail(ESC_EINVAL, "esc_selectivity_shared_async: every predicate must be compiled against the table");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // greedy groups: the union of read columns fits the stage layout
-  int i = 0;
-  while (i < n) {
-    std::vector<int32_t> ucols;
-    int j = i;
-    for (; j < n && j - i < kSharedMaxQueries; ++j) {
-      std::vector<int32_t> add;
-      for (int32_t c : preds[j]->ref_cols)
-        if (std::find(ucols.begin(), ucols.end(), c) == ucols.end()) add.push_back(c);
-      if (ucols.size() + add.size() > (size_t)kMaxRef) break;
-      ucols.insert(ucols.end(), add.begin(), add.end());
+  try {
+    int i = 0;
+    while (i < n) {
+      std::vector<int32_t> ucols;
+      int j = i;
+      for (; j < n && j - i < kSharedMaxQueries; ++j) {
+        std::vector<int32_t> add;
+        for (int32_t c : preds[j]->ref_cols)
+          if (std::find(ucols.begin(), ucols.end(), c) == ucols.end()) add.push_back(c);
+        if (ucols.size() + add.size() > (size_t)kMaxRef) break;
+        ucols.insert(ucols.end(), add.begin(), add.end());
+      }
+      esc_status s = run_shared_group(t, preds + i, j - i, ucols, dev_counts + i, st);
+      if (s != ESC_OK) return s;
+      i = j;
     }
-    esc_status s = run_shared_group(t, preds + i, j - i, ucols, dev_counts + i, st);
-    if (s != ESC_OK) return s;
-    i = j;
+  } catch (const std::bad_alloc &) {
+    return fail(ESC_ENOMEM, "esc_selectivity_shared_async: out of host memory");
   }
   clear_error();
   return ESC_OK;
