@@ -8,15 +8,23 @@
 // [128], W2 [128][128], b2 [128], w3 [128], b3.  The bfloat16 copy has the
 // same layout (its bias entries are unused).
 //
-// Kernel shape: kSets sets of 128 threads per block; in each set, one thread
-// per hidden unit, 8 samples per pass (a block: kSets x 8 samples per pass,
-// one set of weights).  The weight matrices sit in shared memory as bfloat16
-// with padded row strides (66 / 130 elements) so that threads reading their
-// own rows, and threads reading one column, hit distinct banks.  The gradient
-// kernel keeps the block's weight-gradient sums in shared memory (float32);
-// each thread adds the samples of every set into its share of a row (a
-// quarter of the columns), so no two threads update the same sum, and the
-// sums go to the global gradient once, at the end.
+// The matrix products run on the tensor cores (tcgen05.mma, kind::f16): a
+// block takes 128 samples at a time, accumulators and some operands sit in
+// tensor memory.  Nothing loses precision on the way: features and weights are
+// bfloat16 already, and a float32 operand (an activation, a gradient) is the
+// sum of three bfloat16 numbers, its upper, middle and lower 8 significand
+// bits, each multiplied by the other operand in full and accumulated in
+// float32.  The gradient uses that w3 is bfloat16 and that the second layer's
+// gradient is the outer product of dy and w3 under the ReLU mask:
+//   d1 = dy (mask w3) W2,   gW2 = w3 (mask^T (dy z1)),   gb2 = w3 (mask^T dy),
+//   gw3[j] = sum_k W2[j][k] (mask^T (dy z1))[j][k] + b2[j] (mask^T dy)[j],
+// so that only z1, dy z1 and d1 need the split.
+//
+// Shared-memory operands are rows of 128 bytes with 128-byte swizzle (the
+// 16-byte chunk c of row r at c ^ (r % 8)), 64 columns a block of 16 KB per 128
+// rows.  One such block is read along its rows (K-major) or across them
+// (MN-major): X, z1 and the mask need no second copy for the transposed
+// products.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -25,230 +33,614 @@
 #include <string>
 
 #include "esc_internal.h"
+#include "esc_ptx.cuh"
 
 namespace esc {
 
-constexpr int kIn = 64, kH = 128, kS = 8;  // inputs, hidden width, samples per pass and set
-constexpr int kSets = 4;                     // sample sets per block
-constexpr int kMlpThreads = kSets * kH;      // 512
+constexpr int kIn = 64, kH = 128;            // inputs, hidden width
+constexpr int kTileS = 128;                  // samples per tile (rows of an accumulator: one tensor-memory lane each)
+constexpr int kFwdThreads = 256, kGradThreads = 256;   // two warps per 32 lanes of tensor memory: half of the columns each
 constexpr int kW1 = 0, kB1 = kW1 + kH * kIn, kW2 = kB1 + kH, kB2 = kW2 + kH * kH, kW3 = kB2 + kH, kB3 = kW3 + kH;
 constexpr int kParams = kB3 + 1;  // 24961
-constexpr int kT1 = kIn + 4, kT2 = kH + 4;  // padded bf16 row strides (34 and 66 words: 8-byte loads
-                                            // of 16 threads, their rows, hit distinct banks)
-constexpr int kG1 = kIn + 1, kG2 = kH + 1;  // padded float32 row strides of the gradient sums
-static_assert(kH % kSets == 0 && kIn % kSets == 0, "columns split evenly over the sets");
 static_assert(kParams == ESC_MLP_PARAMS, "flat parameter layout");
+static_assert(kW2 % 8 == 0, "16-byte chunks of W2");
+
+constexpr uint32_t kBlock = 128 * 128;       // bytes of a 128-row operand block (64 columns)
+
+// Raised when a wait on the tensor cores gave up (these entry points do not
+// synchronise and have no status to return).
+__device__ ScratchHdr g_mlp_hdr;
 
 __device__ __forceinline__ float bf(const uint16_t v) {
   return __uint_as_float((uint32_t)v << 16);
 }
 
-struct MlpWeights {
-  uint16_t W1[kH * kT1];  // bfloat16
-  uint16_t W2[kH * kT2];
-  float w3[kH], b1[kH], b2[kH];
+// ------------------------------------------------------------------ tcgen05
+__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t cols) {   // one warp
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "r"(cols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t cols) {   // the same warp
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols));
+}
+__device__ __forceinline__ void tc_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// Arrives on the barrier when this thread's earlier products are done.
+__device__ __forceinline__ void tc_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
+               : "memory");
+}
+// Instruction descriptor: float32 accumulators, bfloat16 operands, M = 128;
+// transposed operands are MN-major.
+__device__ __forceinline__ constexpr uint32_t idesc(uint32_t n, bool a_mn, bool b_mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) | ((n >> 3) << 17) |
+         ((128u >> 4) << 24);
+}
+// Shared-memory operand descriptor, 128-byte swizzle: 8-row groups 1024 bytes
+// apart, 64-column blocks (MN-major) kBlock apart.
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
+  return (uint64_t)((addr & 0x3ffffu) >> 4) | ((uint64_t)(kBlock >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
+         (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t id, bool add) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+               "l"(a), "l"(b), "r"(id), "r"((uint32_t)add)
+               : "memory");
+}
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t id, bool add) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+               "r"(a), "l"(b), "r"(id), "r"((uint32_t)add)
+               : "memory");
+}
+// 32 columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+}
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(addr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+
+// Two floats as three pairs of bfloat16: x = hi + mid + lo exactly (a float's
+// 24 significand bits, 8 in each; the low half holds a).  Infinities and NaN
+// stay in hi, their other parts are 0: a truncated remainder has the sign of x,
+// so that for x >= 0 a maximum with 0 clears a NaN.
+template <bool NONNEG>
+__device__ __forceinline__ float finite_part(float r) {
+  return NONNEG ? fmaxf(r, 0.0f) : r == r ? r : 0.0f;
+}
+template <bool NONNEG>
+__device__ __forceinline__ void split3(float2 x, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+  // minus the upper half of a float's bits, as a float
+  auto minus_hi = [](float v) { return __uint_as_float((__float_as_uint(v) & 0xffff0000u) ^ 0x80000000u); };
+  float2 r = __fadd2_rn(x, make_float2(minus_hi(x.x), minus_hi(x.y)));
+  r = make_float2(finite_part<NONNEG>(r.x), finite_part<NONNEG>(r.y));
+  const float2 l = __fadd2_rn(r, make_float2(minus_hi(r.x), minus_hi(r.y)));
+  hi = __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632);
+  mid = __byte_perm(__float_as_uint(r.x), __float_as_uint(r.y), 0x7632);
+  lo = __byte_perm(__float_as_uint(l.x), __float_as_uint(l.y), 0x7632);
+}
+
+// ------------------------------------------------------------------ operands
+// 8 values (16 bytes); plain loads where the array is not 16-byte aligned.
+__device__ __forceinline__ uint4 load8(const uint16_t *p, bool vec) {
+  if (vec) return *reinterpret_cast<const uint4 *>(p);
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = (uint32_t)p[2 * k] | (uint32_t)p[2 * k + 1] << 16;
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ uint8_t *chunk(uint8_t *block, uint32_t row, uint32_t c) {
+  return block + row * 128u + ((c ^ (row & 7u)) << 4);
+}
+
+struct MlpVectors {
+  float b1[kH], b2[kH], w3[kH];
   float b3;
+  float pad[3];
 };
 
-// One set's samples of a pass (16-byte aligned rows: 4 values a load).
-struct alignas(16) MlpSet {
-  float x[kS][kIn];
-  float z1[kS][kH];   // relu(a1)
-  float a1[kS][kH];   // pre-activation; the gradient kernel overwrites it with d loss / d a1
-  float d2[kS][kH];   // d loss / d a2
-  float red[kS][4];   // per-warp partial sums of y
-};
-
-struct MlpSmem {
-  MlpWeights W;
-  MlpSet set[kSets];
-};
-
-struct GradSmem {
-  float gW1[kH * kG1];
-  float gW2[kH * kG2];
-};
-
-__device__ void load_weights(MlpWeights &W, const uint16_t *wbf, const float *pf) {
-  for (int i = threadIdx.x; i < kH * kIn; i += blockDim.x) W.W1[(i / kIn) * kT1 + i % kIn] = wbf[kW1 + i];
-  for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) W.W2[(i / kH) * kT2 + i % kH] = wbf[kW2 + i];
-  for (int i = threadIdx.x; i < kH; i += blockDim.x) {
-    W.w3[i] = bf(wbf[kW3 + i]);
-    W.b1[i] = pf[kB1 + i];
-    W.b2[i] = pf[kB2 + i];
+// W1 (one block) and W2 (two) to shared memory, and the float32 vectors.
+template <int NT>
+__device__ __forceinline__ void load_weights(uint8_t *w1, uint8_t *w2, MlpVectors &V, const uint16_t *wbf, const float *pf) {
+  const bool vec = ((uintptr_t)wbf & 15u) == 0;
+  for (uint32_t i = threadIdx.x; i < kH * kIn / 8; i += NT)
+    *reinterpret_cast<uint4 *>(chunk(w1, i >> 3, i & 7u)) = load8(wbf + kW1 + 8 * i, vec);
+  for (uint32_t i = threadIdx.x; i < kH * kH / 8; i += NT)
+    *reinterpret_cast<uint4 *>(chunk(w2 + ((i >> 3) & 1u) * kBlock, i >> 4, i & 7u)) = load8(wbf + kW2 + 8 * i, vec);
+  for (uint32_t i = threadIdx.x; i < kH; i += NT) {
+    V.b1[i] = pf[kB1 + i];
+    V.b2[i] = pf[kB2 + i];
+    V.w3[i] = bf(wbf[kW3 + i]);
   }
-  if (threadIdx.x == 0) W.b3 = pf[kB3];
+  if (threadIdx.x == 0) V.b3 = pf[kB3];
 }
 
-// Forward of this thread's set (samples s0 .. s0+kS-1, those < B; thread j =
-// hidden unit j of the set): leaves z1, a1 in the set's buffers, returns a2
-// per sample, and the outputs y in S.red[s][0] (valid after the final
-// barrier).  Every thread of the block calls it together (block barriers).
-__device__ void forward_pass(const MlpWeights &W, MlpSet &S, const uint16_t *x, uint64_t B, uint64_t s0,
-                             float (&a2)[kS]) {
-  const int j = threadIdx.x % kH;
-  for (int i = j; i < kS * kIn; i += kH) {
-    const uint64_t s = s0 + i / kIn;
-    S.x[i / kIn][i % kIn] = s < B ? bf(x[s * kIn + i % kIn]) : 0.0f;
+// This thread's chunks of a tile's features (samples past the batch: 0).
+template <int NT>
+__device__ __forceinline__ void load_x(const uint16_t *x, uint64_t B, uint64_t s0, bool vec, uint4 (&r)[1024 / NT]) {
+#pragma unroll
+  for (int q = 0; q < 1024 / NT; ++q) {
+    const uint32_t i = threadIdx.x + q * NT;
+    const uint64_t s = s0 + (i >> 3);
+    r[q] = s < B ? load8(x + s * kIn + 8 * (i & 7u), vec) : make_uint4(0, 0, 0, 0);
   }
-  __syncthreads();
-  float acc[kS];
+}
+template <int NT>
+__device__ __forceinline__ void store_x(uint8_t *xb, const uint4 (&r)[1024 / NT]) {
 #pragma unroll
-  for (int s = 0; s < kS; ++s) acc[s] = W.b1[j];
-  // 4 inputs a step: 4 weights in one 8-byte load, 4 values of each sample in one 16-byte load
-  for (int k = 0; k < kIn; k += 4) {
-    const uint2 w2 = *reinterpret_cast<const uint2 *>(&W.W1[j * kT1 + k]);
-    const float w0 = __uint_as_float(w2.x << 16), w1 = __uint_as_float(w2.x & 0xffff0000u);
-    const float w2f = __uint_as_float(w2.y << 16), w3f = __uint_as_float(w2.y & 0xffff0000u);
+  for (int q = 0; q < 1024 / NT; ++q) {
+    const uint32_t i = threadIdx.x + q * NT;
+    *reinterpret_cast<uint4 *>(chunk(xb, i >> 3, i & 7u)) = r[q];
+  }
+}
+
+// ------------------------------------------------------------------ layers
+// The tensor cores truncate each sum they write, a bias towards 0 that grows
+// with the products added one after the other at full size.  So a float32
+// operand's lower parts are multiplied first, and K is shared among two
+// accumulators (forward) or four (gradient: 128 columns each), summed rounded
+// to nearest here.  How far y is from its 64-bit value (2-norm; features and
+// weights as in training, 31 to 1M samples): 1.5e-7 with the float32
+// multiply-adds these products replace, 2.7e-7 with one accumulator, 1.1e-7
+// with two, 1.0e-7 with four.  The gradient: 1.3e-7 to 3.2e-7 before, 0.8e-7
+// to 2.6e-7 now (32 to 20,000 samples).
+constexpr uint32_t kTmCols = 512;
+
+// a1 = x W1^T: K = 64, 16 (32 bytes) per accumulator.
+__device__ __forceinline__ void issue_layer1(uint32_t tm, uint64_t dx, uint64_t dw1) {
+  for (uint32_t k = 0; k < 4; ++k) mma_ss(tm + 128 * k, dx + 2 * k, dw1 + 2 * k, idesc(kH, false, false), false);
+}
+// a2 = z1 W2^T: K = 128, 32 per accumulator; z1's parts (two blocks each) one
+// after the other, the lower ones first.
+__device__ __forceinline__ void issue_layer2(uint32_t tm, uint64_t dz, uint64_t dw2) {
+  for (int p = 2; p >= 0; --p)
+    for (uint32_t k = 0; k < 8; ++k) {
+      const uint64_t at = (k >> 2) * (kBlock >> 4) + 2 * (k & 3u);
+      mma_ss(tm + 128 * (k >> 1), dz + p * (2 * (kBlock >> 4)) + at, dw2 + at, idesc(kH, false, false), (k & 1u) || p < 2);
+    }
+}
+// 32 columns of the sum of two or four accumulators.
+__device__ __forceinline__ float2 as_float2(uint32_t a, uint32_t b) {
+  return make_float2(__uint_as_float(a), __uint_as_float(b));
+}
+__device__ __forceinline__ void load_sum32(uint32_t addr, float2 (&v)[16]) {
+  uint32_t a[32], b[32];
+  tmem_ld32(addr, a);
+  tmem_ld32(addr + 128, b);
+  tc_wait_ld();
 #pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      const float4 v = *reinterpret_cast<const float4 *>(&S.x[s][k]);
-      acc[s] = fmaf(w0, v.x, acc[s]);
-      acc[s] = fmaf(w1, v.y, acc[s]);
-      acc[s] = fmaf(w2f, v.z, acc[s]);
-      acc[s] = fmaf(w3f, v.w, acc[s]);
+  for (int k = 0; k < 16; ++k) v[k] = __fadd2_rn(as_float2(a[2 * k], a[2 * k + 1]), as_float2(b[2 * k], b[2 * k + 1]));
+}
+__device__ __forceinline__ void load_sum32x4(uint32_t addr, float2 (&v)[16]) {
+  float2 w[16];
+  load_sum32(addr, v);
+  load_sum32(addr + 256, w);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = __fadd2_rn(v[k], w[k]);
+}
+// relu(v + bias) of a pair of units
+__device__ __forceinline__ float2 relu_bias(float2 v, const float *bias) {
+  const float2 s = __fadd2_rn(v, *reinterpret_cast<const float2 *>(bias));
+  return make_float2(fmaxf(s.x, 0.0f), fmaxf(s.y, 0.0f));
+}
+
+// 32 columns of a row of a split operand.
+struct Split32 {
+  uint32_t hi[16], mid[16], lo[16];
+  template <bool NONNEG>
+  __device__ __forceinline__ void make(const float2 *v) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) split3<NONNEG>(v[k], hi[k], mid[k], lo[k]);
+  }
+  // To chunks c .. c + 3 of the row; the parts' blocks lie `dist` apart.
+  __device__ __forceinline__ void store(uint8_t *block, uint32_t dist, uint32_t c, uint32_t row) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint8_t *at = chunk(block, row, c + q);
+      *reinterpret_cast<uint4 *>(at) = make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+      *reinterpret_cast<uint4 *>(at + dist) = make_uint4(mid[4 * q], mid[4 * q + 1], mid[4 * q + 2], mid[4 * q + 3]);
+      *reinterpret_cast<uint4 *>(at + 2 * dist) = make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
     }
   }
-#pragma unroll
-  for (int s = 0; s < kS; ++s) {
-    S.a1[s][j] = acc[s];
-    S.z1[s][j] = fmaxf(acc[s], 0.0f);
+};
+// A quarter (32 units) of a row of R: three parts of two blocks.
+template <bool NONNEG>
+__device__ __forceinline__ void store_split32(uint8_t *r, uint32_t quarter, uint32_t row, const float2 *v) {
+  Split32 s;
+  s.make<NONNEG>(v);
+  s.store(r + (quarter >> 1) * kBlock, 2 * kBlock, 4 * (quarter & 1u), row);
+}
+
+// ------------------------------------------------------------------ forward
+// Two blocks per SM, so that one converts while the other's products run;
+// tiles of 128 samples, two accumulators (tensor memory: 256 columns a block),
+// one for each half of K.  Half of z1 is in shared memory at a time, over the
+// features.  What bounds it: the instructions that split z1 and the waits
+// between products and conversions (0.40 of the issue slots, 2 warps a
+// scheduler and block).  Measured on 1M samples: 1822 us with one thread per
+// hidden unit and float32 multiply-adds, 173 us with one block of 512 threads
+// per SM and four accumulators, 148 us this way.
+struct FwdSmem {
+  static constexpr uint32_t w1 = 0, w2 = kBlock, z = 3 * kBlock, x = z, vec = 6 * kBlock, ypart = vec + sizeof(MlpVectors),
+                            bar = ypart + 4 * kTileS, tmem = bar + 8, total = tmem + 8;
+};
+constexpr uint32_t kFwdCols = 256;
+
+__global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint16_t *x, uint64_t B, const uint16_t *wbf,
+                                                                     const float *pf, float *y) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  MlpVectors &V = *reinterpret_cast<MlpVectors *>(sm + FwdSmem::vec);
+  float *ypart = reinterpret_cast<float *>(sm + FwdSmem::ypart);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + FwdSmem::bar);
+  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + FwdSmem::tmem);
+  uint8_t *Z = sm + FwdSmem::z;
+  const uint32_t warp = threadIdx.x >> 5, half = warp >> 2, row = threadIdx.x & 127u;
+  const bool vec = ((uintptr_t)x & 15u) == 0;
+  uint4 xr[4];
+  load_x<kFwdThreads>(x, B, (uint64_t)blockIdx.x * kTileS, vec, xr);
+  if (warp == 0) tmem_alloc(slot, kFwdCols);
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  load_weights<kFwdThreads>(sm + FwdSmem::w1, sm + FwdSmem::w2, V, wbf, pf);
+  store_x<kFwdThreads>(sm + FwdSmem::x, xr);
+  fence_proxy_async_smem();
+  tc_before_sync();
   __syncthreads();
-#pragma unroll
-  for (int s = 0; s < kS; ++s) acc[s] = W.b2[j];
-  for (int k = 0; k < kH; k += 4) {
-    const uint2 w2 = *reinterpret_cast<const uint2 *>(&W.W2[j * kT2 + k]);
-    const float w0 = __uint_as_float(w2.x << 16), w1 = __uint_as_float(w2.x & 0xffff0000u);
-    const float w2f = __uint_as_float(w2.y << 16), w3f = __uint_as_float(w2.y & 0xffff0000u);
-#pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      const float4 v = *reinterpret_cast<const float4 *>(&S.z1[s][k]);
-      acc[s] = fmaf(w0, v.x, acc[s]);
-      acc[s] = fmaf(w1, v.y, acc[s]);
-      acc[s] = fmaf(w2f, v.z, acc[s]);
-      acc[s] = fmaf(w3f, v.w, acc[s]);
+  tc_after_sync();
+  const uint32_t tm = *slot, lanes = tm + ((warp & 3u) << 21);   // + 32 * (warp % 4) lanes
+  const uint64_t dw1 = sdesc(smem_addr(sm + FwdSmem::w1)), dw2 = sdesc(smem_addr(sm + FwdSmem::w2)),
+                 dx = sdesc(smem_addr(sm + FwdSmem::x)), dz = sdesc(smem_addr(Z));
+  constexpr uint32_t id = idesc(kH, false, false);
+  uint32_t phase = 0;
+  bool ok = true;
+  for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
+    if (threadIdx.x == 0) {   // a1 = x W1^T: K = 64 in steps of 16 (32 bytes)
+      for (uint32_t k = 0; k < 4; ++k) mma_ss(tm + 128 * (k >> 1), dx + 2 * k, dw1 + 2 * k, id, k & 1u);
+      tc_commit(bar);
     }
-  }
-  const float w3 = W.w3[j];
+    ok = mbar_wait(bar, phase, &g_mlp_hdr);
+    phase ^= 1u;
+    tc_after_sync();
+    float2 v[2][16];   // 32 units of either half of z1
 #pragma unroll
-  for (int s = 0; s < kS; ++s) {
-    a2[s] = acc[s];
-    float v = w3 * fmaxf(acc[s], 0.0f);
+    for (int h = 0; h < 2; ++h) {
+      load_sum32(lanes + 64 * h + 32 * half, v[h]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((j & 31) == 0) S.red[s][j >> 5] = v;
-  }
-  __syncthreads();
-  if (j < kS) S.red[j][0] = S.red[j][0] + S.red[j][1] + S.red[j][2] + S.red[j][3] + W.b3;
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(kMlpThreads, 2) mlp_forward_kernel(const uint16_t *x, uint64_t B, const uint16_t *wbf,
-                                                                  const float *pf, float *y) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  MlpSmem &S = *reinterpret_cast<MlpSmem *>(smem);
-  const int q = threadIdx.x / kH, j = threadIdx.x % kH;
-  load_weights(S.W, wbf, pf);
-  __syncthreads();
-  // block-uniform trip count: every set of the block passes together
-  for (uint64_t c0 = (uint64_t)blockIdx.x * (kSets * kS); c0 < B; c0 += (uint64_t)gridDim.x * (kSets * kS)) {
-    const uint64_t s0 = c0 + (uint64_t)q * kS;
-    float a2[kS];
-    forward_pass(S.W, S.set[q], x, B, s0, a2);
-    if (j < kS && s0 + j < B) y[s0 + j] = S.set[q].red[j][0];
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(kMlpThreads) mlp_grad_kernel(const uint16_t *x, const float *t, uint64_t B,
-                                                               const uint16_t *wbf, const float *pf, float *grad,
-                                                               float *loss_sum) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  MlpSmem &S = *reinterpret_cast<MlpSmem *>(smem);
-  GradSmem &G = *reinterpret_cast<GradSmem *>(smem + ((sizeof(MlpSmem) + 15) & ~(size_t)15));
-  const int q = threadIdx.x / kH, j = threadIdx.x % kH;
-  MlpSet &me = S.set[q];
-  load_weights(S.W, wbf, pf);
-  for (int i = threadIdx.x; i < kH * kG1; i += blockDim.x) G.gW1[i] = 0.0f;
-  for (int i = threadIdx.x; i < kH * kG2; i += blockDim.x) G.gW2[i] = 0.0f;
-  __syncthreads();
-  float gb1 = 0.0f, gb2 = 0.0f, gw3 = 0.0f, gb3 = 0.0f, lsum = 0.0f;
-  const float inv_b = 2.0f / (float)B;
-  constexpr int kC2 = kH / kSets, kC1 = kIn / kSets;  // this thread's columns of a gradient row
-  for (uint64_t c0 = (uint64_t)blockIdx.x * (kSets * kS); c0 < B; c0 += (uint64_t)gridDim.x * (kSets * kS)) {
-    const uint64_t s0 = c0 + (uint64_t)q * kS;
-    float a2[kS];
-    forward_pass(S.W, me, x, B, s0, a2);
-    // output layer and second hidden layer: thread j owns unit j of its set's samples
-    const float w3 = S.W.w3[j];
+      for (int k = 0; k < 16; ++k) v[h][k] = relu_bias(v[h][k], V.b1 + 64 * h + 32 * half + 2 * k);
+    }
 #pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      const bool ok = s0 + s < B;
-      const float e = ok ? me.red[s][0] - t[s0 + s] : 0.0f;
-      const float dy = e * inv_b;
-      if (j == 0) {
-        lsum += e * e;
-        gb3 += dy;
+    for (int h = 0; h < 2; ++h) {
+      Split32 z;
+      z.make<true>(v[h]);
+      if (h == 1) {   // the first half's products have read Z
+        ok = mbar_wait(bar, phase, &g_mlp_hdr) && ok;
+        phase ^= 1u;
       }
-      const float z2 = fmaxf(a2[s], 0.0f);
-      gw3 = fmaf(dy, z2, gw3);
-      const float d2 = a2[s] > 0.0f ? dy * w3 : 0.0f;
-      me.d2[s][j] = d2;
-      gb2 += d2;
+      z.store(Z, kBlock, 4 * half, row);
+      if (h == 0) load_x<kFwdThreads>(x, B, s0 + (uint64_t)gridDim.x * kTileS, vec, xr);   // the next tile's features
+      fence_proxy_async_smem();
+      tc_before_sync();
+      __syncthreads();
+      if (threadIdx.x == 0) {   // a2 = z1 W2^T, the lower parts first
+        tc_after_sync();
+        for (int p = 2; p >= 0; --p)
+          for (uint32_t k = 0; k < 4; ++k)
+            mma_ss(tm + 128 * h, dz + p * (kBlock >> 4) + 2 * k, dw2 + h * (kBlock >> 4) + 2 * k, id, p < 2 || k > 0);
+        tc_commit(bar);
+      }
     }
-    __syncthreads();
-    // row j of W2's gradient, columns q*kC2 .. q*kC2+kC2-1, over every set's samples
-    for (int kk = 0; kk < kC2; ++kk) {
-      const int k = q * kC2 + kk;
-      float g = G.gW2[j * kG2 + k];
+    ok = mbar_wait(bar, phase, &g_mlp_hdr) && ok;
+    phase ^= 1u;
+    tc_after_sync();
+    store_x<kFwdThreads>(sm + FwdSmem::x, xr);
+    fence_proxy_async_smem();
+    float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
 #pragma unroll
-      for (int p = 0; p < kSets; ++p)
+    for (int h = 0; h < 2; ++h) {
+      load_sum32(lanes + 64 * half + 32 * h, v[h]);
 #pragma unroll
-        for (int s = 0; s < kS; ++s) g = fmaf(S.set[p].d2[s][j], S.set[p].z1[s][k], g);
-      G.gW2[j * kG2 + k] = g;
+      for (int k = 0; k < 16; ++k) {
+        const int j = 64 * half + 32 * h + 2 * k;
+        acc[k & 1] = __ffma2_rn(*reinterpret_cast<const float2 *>(V.w3 + j), relu_bias(v[h][k], V.b2 + j), acc[k & 1]);
+      }
     }
-    // first hidden layer: thread k owns unit k of its set's samples (column k of W2)
-    const int k = j;
-    float d1[kS];
-#pragma unroll
-    for (int s = 0; s < kS; ++s) d1[s] = 0.0f;
-    for (int i = 0; i < kH; ++i) {
-      const float w = bf(S.W.W2[i * kT2 + k]);
-#pragma unroll
-      for (int s = 0; s < kS; ++s) d1[s] = fmaf(w, me.d2[s][i], d1[s]);
-    }
-#pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      d1[s] = me.a1[s][k] > 0.0f ? d1[s] : 0.0f;
-      gb1 += d1[s];
-    }
-    __syncthreads();  // every thread has read its a1 before any overwrites it
-#pragma unroll
-    for (int s = 0; s < kS; ++s) me.a1[s][k] = d1[s];  // a1 now holds d loss / d a1
-    __syncthreads();
-    // row k of W1's gradient, columns q*kC1 .. q*kC1+kC1-1, over every set's samples
-    for (int mm = 0; mm < kC1; ++mm) {
-      const int m = q * kC1 + mm;
-      float g = G.gW1[k * kG1 + m];
-#pragma unroll
-      for (int p = 0; p < kSets; ++p)
-#pragma unroll
-        for (int s = 0; s < kS; ++s) g = fmaf(S.set[p].a1[s][k], S.set[p].x[s][m], g);
-      G.gW1[k * kG1 + m] = g;
-    }
-    __syncthreads();
+    const float part = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+    if (half == 1) ypart[row] = part;
+    tc_before_sync();
+    if (!__syncthreads_and(ok)) break;   // a wait gave up (recorded): the whole block leaves
+    tc_after_sync();
+    if (half == 0 && s0 + row < B) y[s0 + row] = part + ypart[row] + V.b3;   // (ypart is written again two barriers later)
   }
-  // add this block's sums to the global gradient
-  for (int i = threadIdx.x; i < kH * kIn; i += blockDim.x) atomicAdd(&grad[kW1 + i], G.gW1[(i / kIn) * kG1 + i % kIn]);
-  for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) atomicAdd(&grad[kW2 + i], G.gW2[(i / kH) * kG2 + i % kH]);
-  atomicAdd(&grad[kB1 + j], gb1);
-  atomicAdd(&grad[kB2 + j], gb2);
-  atomicAdd(&grad[kW3 + j], gw3);
-  if (j == 0) {
-    atomicAdd(&grad[kB3], gb3);
-    atomicAdd(loss_sum, lsum);
+  __syncthreads();
+  if (warp == 0) tmem_free(tm, kFwdCols);
+}
+
+// ------------------------------------------------------------------ gradient
+// One block per SM, tiles of 128 samples; a tile's sums go to the global
+// gradient by themselves.  Tensor memory: a1 and a2 take all 512 columns (four
+// accumulators); then 0..255 two accumulators of d1 and 448 mask w3 (d1's left
+// operand); when d1 has been read, 0, 128 and 256 three accumulators of gW2 /
+// w3 (rows: units j), 384 gb2 / w3 and gb1 (products with the block E), 448
+// gW1 (rows: units k).
+// E (64 columns): columns 1..3 hold the three parts of dy while the mask is
+// multiplied with it, column 0 then 1 for gb1.
+// R holds z1, then dy z1, then d1, in three parts of two blocks.
+// What bounds it at 4096 samples (32 tiles on 32 SMs): the chain of products
+// and conversions of one tile and the loading of weights.  A training step
+// (two fills, this, Adam; bound by the host's launches up to 20,000 samples):
+// 4096 samples 51.7 -> 35.8 us, 20,000 162 -> 45, 65,536 417 -> 80.
+constexpr uint32_t kTgB = 384, kTm = 448, kTgW1 = 448;
+struct GradSmem {
+  static constexpr uint32_t w1 = 0, w2 = kBlock, x = 3 * kBlock, e = 4 * kBlock, mask = 5 * kBlock, r = 7 * kBlock,
+                            vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * kTileS, tmem = bar + 16,
+                            total = tmem + 16;
+};
+
+__device__ __forceinline__ void add4(float *p, float a, float b, float c, float d, bool vec) {
+  if (vec) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+  } else {
+    atomicAdd(p, a);
+    atomicAdd(p + 1, b);
+    atomicAdd(p + 2, c);
+    atomicAdd(p + 3, d);
   }
+}
+
+__global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_t *x, const float *t, uint64_t B,
+                                                                   const uint16_t *wbf, const float *pf, float *grad,
+                                                                   float *loss_sum) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  MlpVectors &V = *reinterpret_cast<MlpVectors *>(sm + GradSmem::vec);
+  float *part = reinterpret_cast<float *>(sm + GradSmem::part);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [2]
+  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + GradSmem::tmem);
+  uint8_t *R = sm + GradSmem::r, *E = sm + GradSmem::e, *mask = sm + GradSmem::mask;
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, half = warp >> 2, row = threadIdx.x & 127u;
+  const bool vec = ((uintptr_t)x & 15u) == 0, gvec = ((uintptr_t)grad & 15u) == 0;
+  uint4 xr[4];
+  load_x<kGradThreads>(x, B, (uint64_t)blockIdx.x * kTileS, vec, xr);
+  if (warp == 0) tmem_alloc(slot, kTmCols);
+  if (threadIdx.x == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  load_weights<kGradThreads>(sm + GradSmem::w1, sm + GradSmem::w2, V, wbf, pf);
+#pragma unroll
+  for (uint32_t c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(chunk(E, row, 4 * half + c)) = make_uint4(0, 0, 0, 0);
+  store_x<kGradThreads>(sm + GradSmem::x, xr);
+  fence_proxy_async_smem();
+  tc_before_sync();
+  __syncthreads();
+  tc_after_sync();
+  const uint32_t tm = *slot, lanes = tm + ((warp & 3u) << 21);
+  const uint64_t dw1 = sdesc(smem_addr(sm + GradSmem::w1)), dw2 = sdesc(smem_addr(sm + GradSmem::w2)),
+                 dx = sdesc(smem_addr(sm + GradSmem::x)), de = sdesc(smem_addr(E)), dm = sdesc(smem_addr(mask)),
+                 dr = sdesc(smem_addr(R));
+  constexpr uint32_t kPart = 2 * (kBlock >> 4);   // descriptor distance of two parts of R
+  constexpr uint32_t kRows16 = 2048 >> 4;         // of 16 rows (MN-major: a step of K)
+  uint32_t ph0 = 0, ph1 = 0;
+  bool ok = true;
+  float lsum = 0.0f, gb3 = 0.0f;
+  const float inv_b = 2.0f / (float)B;
+  for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
+    if (threadIdx.x == 0) {
+      issue_layer1(tm, dx, dw1);
+      tc_commit(&bar[0]);
+    }
+    const float target = s0 + row < B ? t[s0 + row] : 0.0f;
+    ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr);
+    ph0 ^= 1u;
+    tc_after_sync();
+    float2 z1[32];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 v[16];
+      load_sum32x4(lanes + 64 * half + 32 * h, v);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) z1[16 * h + k] = relu_bias(v[k], V.b1 + 64 * half + 32 * h + 2 * k);
+      store_split32<true>(R, 2 * half + h, row, z1 + 16 * h);
+    }
+    fence_proxy_async_smem();
+    tc_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_after_sync();
+      issue_layer2(tm, dr, dw2);
+      tc_commit(&bar[0]);
+    }
+    ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
+    ph0 ^= 1u;
+    tc_after_sync();
+    float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+    uint32_t mw[2][16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // 32 units at a time: y, the mask, mask w3
+      float2 v[16];
+      load_sum32x4(lanes + 64 * half + 32 * h, v);
+      uint32_t mk[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int j = 64 * half + 32 * h + 2 * k;
+        const float2 w = *reinterpret_cast<const float2 *>(V.w3 + j), z2 = relu_bias(v[k], V.b2 + j);
+        acc[k & 1] = __ffma2_rn(w, z2, acc[k & 1]);
+        const uint32_t on = (z2.x > 0.0f ? 0x0000ffffu : 0u) | (z2.y > 0.0f ? 0xffff0000u : 0u);
+        mk[k] = on & 0x3f803f80u;   // 1.0 in bfloat16
+        mw[h][k] = on & __byte_perm(__float_as_uint(w.x), __float_as_uint(w.y), 0x7632);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<uint4 *>(chunk(mask + half * kBlock, row, 4 * h + c)) =
+            make_uint4(mk[4 * c], mk[4 * c + 1], mk[4 * c + 2], mk[4 * c + 3]);
+    }
+    // y of the row: the two halves' sums
+    const float mine = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+    if (half == 1) part[row] = mine;
+    tc_before_sync();
+    __syncthreads();   // (a2 has been read by all: its columns are free)
+    tc_after_sync();
+    tmem_st16(lanes + kTm + 32 * half, mw[0]);
+    tmem_st16(lanes + kTm + 32 * half + 16, mw[1]);
+    if (half == 0) {
+      const float e = s0 + row < B ? mine + part[row] + V.b3 - target : 0.0f;
+      part[row] = e * inv_b;
+      lsum = fmaf(e, e, lsum);
+      gb3 += e * inv_b;
+    }
+    tc_wait_st();
+    tc_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_after_sync();
+      for (uint32_t k = 0; k < 8; ++k)   // d1 = (mask w3) W2
+        mma_ts(tm + 128 * (k >> 2), tm + kTm + 8 * k, dw2 + k * kRows16, idesc(kH, false, true), (k & 3u) > 0);
+      tc_commit(&bar[0]);
+    }
+    const float dy = part[row];   // (0 past the batch: such a row adds nothing)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // (layer 2's products have read z1)
+      float2 v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = make_float2(dy * z1[16 * h + k].x, dy * z1[16 * h + k].y);
+      store_split32<false>(R, 2 * half + h, row, v);
+    }
+    if (half == 0) {
+      uint32_t hi, mid, lo;
+      split3<false>(make_float2(dy, 0.0f), hi, mid, lo);
+      *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(hi << 16, mid | lo << 16, 0, 0);
+    }
+    fence_proxy_async_smem();
+    ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
+    ph0 ^= 1u;
+    tc_after_sync();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 d[16];
+      load_sum32(lanes + 64 * half + 32 * h, d);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {   // d1
+        float2 &z = z1[16 * h + k];
+        z = make_float2(z.x > 0.0f ? dy * d[k].x : 0.0f, z.y > 0.0f ? dy * d[k].y : 0.0f);
+      }
+    }
+    tc_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_after_sync();
+      for (int p = 2; p >= 0; --p)         // mask^T (dy z1): every third 16 samples per accumulator
+        for (uint32_t k = 0; k < 8; ++k)
+          mma_ss(tm + 128 * (k % 3), dm + k * kRows16, dr + p * kPart + k * kRows16, idesc(kH, true, true), p < 2 || k > 2);
+      for (uint32_t k = 0; k < 8; ++k)     // mask^T E
+        mma_ss(tm + kTgB, dm + k * kRows16, de + k * kRows16, idesc(64, true, true), k > 0);
+      tc_commit(&bar[1]);
+    }
+    load_x<kGradThreads>(x, B, s0 + (uint64_t)gridDim.x * kTileS, vec, xr);
+    ok = mbar_wait(&bar[1], ph1, &g_mlp_hdr) && ok;   // R and E are free
+    ph1 ^= 1u;
+    tc_after_sync();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) store_split32<false>(R, 2 * half + h, row, z1 + 16 * h);
+    if (half == 0) *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(0x3f80u, 0, 0, 0);
+    fence_proxy_async_smem();
+    tc_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_after_sync();
+      for (int p = 2; p >= 0; --p)
+        for (uint32_t k = 0; k < 8; ++k) {
+          const uint64_t a = dr + p * kPart + k * kRows16;
+          mma_ss(tm + kTgW1, a, dx + k * kRows16, idesc(kIn, true, true), p < 2 || k > 0);   // d1^T x
+          mma_ss(tm + kTgB, a, de + k * kRows16, idesc(64, true, true), true);               // d1^T E
+        }
+      tc_commit(&bar[0]);
+    }
+    // meanwhile gW2 goes out: row j is this thread's lane
+    const float w3 = V.w3[row];
+    float2 dot = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 v[16];
+      load_sum32(lanes + 64 * half + 32 * h, v);
+      {
+        uint32_t a[32];
+        tmem_ld32(lanes + 256 + 64 * half + 32 * h, a);
+        tc_wait_ld();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = __fadd2_rn(v[k], as_float2(a[2 * k], a[2 * k + 1]));
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(chunk(sm + GradSmem::w2 + half * kBlock, row, 4 * h + c));
+        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+        const float2 *g = v + 4 * c;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          dot = __ffma2_rn(as_float2(ww[k] << 16, ww[k] & 0xffff0000u), g[k], dot);
+        float *p = grad + kW2 + row * kH + 64 * half + 32 * h + 8 * c;
+        add4(p, w3 * g[0].x, w3 * g[0].y, w3 * g[1].x, w3 * g[1].y, gvec);
+        add4(p + 4, w3 * g[2].x, w3 * g[2].y, w3 * g[3].x, w3 * g[3].y, gvec);
+      }
+    }
+    ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
+    ph0 ^= 1u;
+    tc_after_sync();
+    {
+      uint32_t a[32];
+      tmem_ld32(lanes + kTgW1 + 32 * half, a);
+      tc_wait_ld();
+#pragma unroll
+      for (int k = 0; k < 32; k += 4)
+        add4(grad + kW1 + row * kIn + 32 * half + k, __uint_as_float(a[k]), __uint_as_float(a[k + 1]),
+             __uint_as_float(a[k + 2]), __uint_as_float(a[k + 3]), gvec);
+      float gd = 0.0f;   // mask^T dy
+      if (half == 0) {
+        tmem_ld32(lanes + kTgB, a);
+        tc_wait_ld();
+        gd = (__uint_as_float(a[1]) + __uint_as_float(a[2])) + __uint_as_float(a[3]);
+        atomicAdd(&grad[kB1 + row], __uint_as_float(a[0]));
+        atomicAdd(&grad[kB2 + row], w3 * gd);
+      }
+      atomicAdd(&grad[kW3 + row], fmaf(V.b2[row], gd, dot.x + dot.y));   // each half its units
+    }
+    store_x<kGradThreads>(sm + GradSmem::x, xr);
+    fence_proxy_async_smem();
+    tc_before_sync();
+    ok = __syncthreads_and(ok) != 0;
+    if (!ok) break;   // a wait gave up (recorded): the whole block leaves
+    tc_after_sync();
+  }
+  if (half == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lsum += __shfl_xor_sync(FULL, lsum, o);
+      gb3 += __shfl_xor_sync(FULL, gb3, o);
+    }
+    if (lane == 0) {
+      atomicAdd(&grad[kB3], gb3);
+      atomicAdd(loss_sum, lsum);
+    }
+  }
+  __syncthreads();
+  if (warp == 0) tmem_free(tm, kTmCols);
 }
 
 __global__ void adam_kernel(float *p, uint16_t *wbf, const float *g, float *m, float *v, uint64_t n, float lr,
@@ -266,9 +658,6 @@ __global__ void adam_kernel(float *p, uint16_t *wbf, const float *g, float *m, f
   }
 }
 
-size_t fwd_smem() { return sizeof(MlpSmem); }
-size_t grad_smem() { return ((sizeof(MlpSmem) + 15) & ~(size_t)15) + sizeof(GradSmem); }
-
 }  // namespace esc
 
 using namespace esc;
@@ -280,13 +669,12 @@ using namespace esc;
   } while (0)
 
 namespace {
-// Blocks for a batch: one per kSets x kS samples, at most `per_sm` per SM.
+// Blocks for a batch: one per tile of samples, at most `per_sm` per SM.
 int grid_for(uint64_t B, int per_sm) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t chunks = (B + kSets * kS - 1) / (kSets * kS);
-  return (int)std::max<uint64_t>(1, std::min<uint64_t>(chunks, (uint64_t)sms * per_sm));
+  return (int)std::max<uint64_t>(1, std::min<uint64_t>((B + kTileS - 1) / kTileS, (uint64_t)sms * per_sm));
 }
 }  // namespace
 
@@ -297,9 +685,8 @@ esc_status esc_mlp_forward(const uint16_t *x_bf16, uint64_t batch, const uint16_
   ESC_RANGE("esc_mlp_forward");
   if (batch == 0) return ESC_OK;
   if (!x_bf16 || !w_bf16 || !params || !y) return fail(ESC_EINVAL, "esc_mlp_forward: NULL argument");
-  ESC_MLP_CK(cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem()));
-  // two blocks per SM: the weights (bfloat16) and the sets' buffers take 110 KB
-  mlp_forward_kernel<<<grid_for(batch, 2), kMlpThreads, fwd_smem(), static_cast<cudaStream_t>(stream)>>>(
+  ESC_MLP_CK(cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem::total));
+  mlp_forward_kernel<<<grid_for(batch, 2), kFwdThreads, FwdSmem::total, static_cast<cudaStream_t>(stream)>>>(
       x_bf16, batch, w_bf16, params, y);
   ESC_MLP_CK(cudaGetLastError());
   clear_error();
@@ -312,8 +699,8 @@ esc_status esc_mlp_grad(const uint16_t *x_bf16, const float *target, uint64_t ba
   if (batch == 0) return ESC_OK;
   if (!x_bf16 || !target || !w_bf16 || !params || !grad || !loss_sum)
     return fail(ESC_EINVAL, "esc_mlp_grad: NULL argument");
-  ESC_MLP_CK(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem()));
-  mlp_grad_kernel<<<grid_for(batch, 1), kMlpThreads, grad_smem(), static_cast<cudaStream_t>(stream)>>>(
+  ESC_MLP_CK(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem::total));
+  mlp_grad_kernel<<<grid_for(batch, 1), kGradThreads, GradSmem::total, static_cast<cudaStream_t>(stream)>>>(
       x_bf16, target, batch, w_bf16, params, grad, loss_sum);
   ESC_MLP_CK(cudaGetLastError());
   clear_error();
