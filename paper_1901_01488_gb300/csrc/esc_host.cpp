@@ -800,6 +800,7 @@ void fill_query_program(const esc_pred *p, Query *q) {
   }
   for (int i = 0; i < p->ninstr; ++i) q->code[i] = p->code[i];
   for (size_t i = 0; i < p->pool.size(); ++i) q->pool[i] = p->pool[i];
+  q->npool = (uint32_t)p->pool.size();
 }
 
 std::atomic<int32_t> g_fail_allocs{0};

@@ -1,6 +1,7 @@
 // Internal layout shared by the host compiler (esc_host.cpp) and the CUDA
 // kernels (esc_scan.cu, esc_semijoin.cu).  Not part of the public ABI.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 #include <string>
 #include <vector>
@@ -125,7 +126,8 @@ struct Query {
   uint32_t unit_big;      // work units 0..unit_big-1 hold unit_tiles tiles, the later ones one tile
   uint32_t wunit_groups;  // groups per compaction unit (1..kMaxUnitRows / kGroup)
   uint32_t wunit_recip;   // ceil(2^32 / wunit_groups), 0 for one group: group -> unit by a multiply-high
-  uint32_t pad2[2];
+  uint32_t npool;         // constants in use
+  uint32_t pad2;
   const uint8_t *ref_ptr[kMaxRef];
   const uint8_t *proj_ptr[kMaxProj];
   void *out_proj[kMaxProj];
@@ -141,6 +143,13 @@ struct Query {
   int64_t pool[kMaxPool];
 };
 static_assert(sizeof(Query) % 16 == 0, "Query is copied with 16-byte vectors");
+static_assert(offsetof(Query, code) % 16 == 0 && sizeof(Instr) == 32, "and only as far as it is used");
+
+// The count word of a single sub-query's scan: the blocks' counts in the low
+// 40 bits, the number of finished blocks above, and a flag that some block
+// gave up (its status is in the header).
+constexpr int kDoneShift = 40;
+constexpr unsigned long long kCountMask = (1ull << kDoneShift) - 1, kGaveUp = 1ull << 63;
 
 // Per-launch header in device scratch memory (zeroed before launch).
 struct ScratchHdr {
@@ -149,10 +158,27 @@ struct ScratchHdr {
   unsigned int abort;    // set together with status; everyone stops working
   unsigned int site;     // checked build: where the first out-of-range index was found
   unsigned long long value;  // checked build: that index
-  unsigned int warps_done;   // consumer warps of the scan that have finished (see Launch::count_out)
+  unsigned int blocks_done;  // blocks of a semi-join that have finished
   unsigned int pad;
 };
 static_assert(sizeof(ScratchHdr) == 32, "ScratchHdr layout");
+
+// What a synchronous call needs on the device beside its outputs.  Slots live
+// in the library's device image, all zero when free: the launch's last block
+// reports to the host (HostResult, pinned memory) and clears the slot, so that
+// such a call neither zeroes nor copies anything.
+struct alignas(256) CallSlot {
+  ScratchHdr hdr;
+  unsigned long long count;
+  unsigned long long hist[16];   // semi-join bins
+};
+struct alignas(64) HostResult {
+  unsigned long long seq;        // written last: the number of the call that the rest belongs to
+  unsigned long long count;
+  unsigned int status;           // as in ScratchHdr
+  unsigned int pad;
+  unsigned long long hist[16];
+};
 
 #ifdef __CUDACC__
 // Checked build (-DESC_CHECKED, libesc_checked.so; the stand-in for a memory
@@ -210,6 +236,20 @@ esc_status device_status(const ScratchHdr &h, const char *where);
 // Test hook: true when a device allocation of the library is to fail
 // (esc_debug_fail_allocs counts them down).
 bool inject_alloc_failure();
+// A free slot of the current device for one synchronous call on `stream`
+// (esc_scan.cu): null when all are in use or the stream is being captured; the
+// call then allocates scratch.  give_slot returns it when the launch is known
+// to have completed; a slot whose launch failed is not used again.
+struct SlotRef {
+  CallSlot *dev = nullptr;
+  HostResult *host = nullptr;      // the host's address
+  HostResult *host_dev = nullptr;  // the device's address of the same memory
+  unsigned long long seq = 0;      // this call's number
+  int device = 0, index = -1;
+};
+bool take_slot(void *stream, SlotRef *out);
+bool poll_slot(const SlotRef &s);   // waits for its report, at most 2 ms
+void give_slot(const SlotRef &s);
 // A named range on the calling host thread for timeline tools (NVTX; with
 // no tool attached a push or pop is a call through a no-op pointer).  Every
 // public entry point that launches GPU work opens one.

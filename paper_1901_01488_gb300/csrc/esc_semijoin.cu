@@ -41,7 +41,9 @@ struct SjParams {
   int32_t ndims;
   uint32_t nrows;
   unsigned long long *hist;            // 16 bins, zeroed
-  ScratchHdr *hdr;                     // launch header (zeroed): the checked build's findings
+  ScratchHdr *hdr;                     // launch header (zeroed): blocks done, the checked build's findings
+  HostResult *result;                  // hist and hdr are a call slot: the last block reports here and clears them
+  unsigned long long seq;              // for result
   uint32_t smem_words;                 // shared-memory words the launch has (checked build)
 };
 
@@ -180,6 +182,26 @@ __global__ void __launch_bounds__(kSjThreads, 1) semijoin_kernel(const __grid_co
   flush(lo, hi, bins);
   __syncthreads();
   if (threadIdx.x < 16 && bins[threadIdx.x]) atomicAdd(&P.hist[threadIdx.x], (unsigned long long)bins[threadIdx.x]);
+  if (P.result && threadIdx.x < 32) {
+    __threadfence();
+    __syncwarp();
+    uint32_t last = 0;
+    if (threadIdx.x == 0) last = atomicAdd(&P.hdr->blocks_done, 1u) == gridDim.x - 1u;
+    if (__shfl_sync(0xffffffffu, last, 0)) {
+      __threadfence();
+      if (threadIdx.x < 16) {
+        P.result->hist[threadIdx.x] = atomicAdd(&P.hist[threadIdx.x], 0ull);
+        P.hist[threadIdx.x] = 0;
+      }
+      if (threadIdx.x == 0) {
+        P.result->status = 0;   // (the release build's kernel raises none)
+        *P.hdr = ScratchHdr{};
+      }
+      __threadfence_system();   // the slot is clear before the host can know
+      __syncwarp();
+      if (threadIdx.x == 0) *(volatile unsigned long long *)&P.result->seq = P.seq;
+    }
+  }
 }
 
 template <int ND, int NS>
@@ -267,13 +289,27 @@ extern "C" esc_status esc_semijoin_counts(const esc_table *fact, const char *con
     }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // a call slot, or scratch from the library's device pool (memory stays
+  // reserved between calls): 16 bins, then the launch header
   void *mem = nullptr;
-  // the library's device pool (memory stays reserved between calls): 16
-  // bins, then the launch header
-  if (esc_status as = alloc_async(&mem, 16 * 8 + sizeof(ScratchHdr), st); as != ESC_OK) return as;
-  cudaError_t e = cudaMemsetAsync(mem, 0, 16 * 8 + sizeof(ScratchHdr), st);
-  P.hist = static_cast<unsigned long long *>(mem);
-  P.hdr = reinterpret_cast<ScratchHdr *>(static_cast<uint8_t *>(mem) + 16 * 8);
+  SlotRef slot;
+  const bool in_slot = take_slot(st, &slot);
+  cudaError_t e = cudaSuccess;
+  if (in_slot) {
+    if (inject_alloc_failure()) {
+      give_slot(slot);
+      return fail(ESC_ENOMEM, "device scratch allocation: injected failure (esc_debug_fail_allocs)");
+    }
+    P.hist = slot.dev->hist;
+    P.hdr = &slot.dev->hdr;
+    P.result = slot.host_dev;
+    P.seq = slot.seq;
+  } else {
+    if (esc_status as = alloc_async(&mem, 16 * 8 + sizeof(ScratchHdr), st); as != ESC_OK) return as;
+    e = cudaMemsetAsync(mem, 0, 16 * 8 + sizeof(ScratchHdr), st);
+    P.hist = static_cast<unsigned long long *>(mem);
+    P.hdr = reinterpret_cast<ScratchHdr *>(static_cast<uint8_t *>(mem) + 16 * 8);
+  }
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -294,10 +330,16 @@ extern "C" esc_status esc_semijoin_counts(const esc_table *fact, const char *con
     ScratchHdr hdr;
   } back;
   unsigned long long *h = back.h;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&back, mem, sizeof back, cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(mem, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && !in_slot) e = cudaMemcpyAsync(&back, mem, sizeof back, cudaMemcpyDeviceToHost, st);
+  if (mem) cudaFreeAsync(mem, st);
+  if (e == cudaSuccess && !(in_slot && poll_slot(slot))) e = cudaStreamSynchronize(st);
+  // (after a failure the slot stays taken: its launch may still be running)
   if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_semijoin_counts: ") + cudaGetErrorString(e));
+  if (in_slot) {
+    std::memcpy(back.h, slot.host->hist, sizeof back.h);
+    back.hdr.status = slot.host->status;
+    give_slot(slot);
+  }
   if (back.hdr.status != 0) return device_status(back.hdr, "esc_semijoin_counts");
   // bins are in probe order (bit i = dimension order[i]): back to the caller's bits
   const uint32_t nsub = 1u << ndims;

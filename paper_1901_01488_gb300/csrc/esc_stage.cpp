@@ -23,14 +23,6 @@ struct Pool {
   StageBlock small[kSmall], large[kLarge];
 } g_pool[kDevices];
 
-// Event and allocation calls are refused to every thread while one captures a
-// stream in global mode; these touch no capturing stream.
-struct RelaxedCapture {
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
-
 StageBlock *acquire(size_t bytes, cudaStream_t st) {
   if (bytes <= kInlineBytes || bytes > kLargeBytes) return nullptr;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

@@ -15,6 +15,14 @@
 
 namespace esc {
 
+// Event and allocation calls are refused to every thread while one captures a
+// stream in global mode; these touch no capturing stream.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 struct StageBlock;
 
 class HostStage {
