@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include "esc_internal.h"
@@ -669,12 +670,25 @@ using namespace esc;
   } while (0)
 
 namespace {
-// Blocks for a batch: one per tile of samples, at most `per_sm` per SM.
-int grid_for(uint64_t B, int per_sm) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return (int)std::max<uint64_t>(1, std::min<uint64_t>((B + kTileS - 1) / kTileS, (uint64_t)sms * per_sm));
+// Blocks for a batch: one per tile of samples, at most `per_sm` per SM; the
+// kernels' attributes are set on a device's first call.
+cudaError_t grid_for(uint64_t B, int per_sm, int *grid) {
+  static std::once_flag once[64];
+  static cudaError_t attr[64];
+  static int sms[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [&] {
+    attr[dev] = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+    if (attr[dev] == cudaSuccess)
+      attr[dev] = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem::total);
+    if (attr[dev] == cudaSuccess)
+      attr[dev] = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem::total);
+  });
+  *grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((B + kTileS - 1) / kTileS, (uint64_t)sms[dev] * per_sm));
+  return attr[dev];
 }
 }  // namespace
 
@@ -685,8 +699,9 @@ esc_status esc_mlp_forward(const uint16_t *x_bf16, uint64_t batch, const uint16_
   ESC_RANGE("esc_mlp_forward");
   if (batch == 0) return ESC_OK;
   if (!x_bf16 || !w_bf16 || !params || !y) return fail(ESC_EINVAL, "esc_mlp_forward: NULL argument");
-  ESC_MLP_CK(cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem::total));
-  mlp_forward_kernel<<<grid_for(batch, 2), kFwdThreads, FwdSmem::total, static_cast<cudaStream_t>(stream)>>>(
+  int grid = 0;
+  ESC_MLP_CK(grid_for(batch, 2, &grid));
+  mlp_forward_kernel<<<grid, kFwdThreads, FwdSmem::total, static_cast<cudaStream_t>(stream)>>>(
       x_bf16, batch, w_bf16, params, y);
   ESC_MLP_CK(cudaGetLastError());
   clear_error();
@@ -699,8 +714,9 @@ esc_status esc_mlp_grad(const uint16_t *x_bf16, const float *target, uint64_t ba
   if (batch == 0) return ESC_OK;
   if (!x_bf16 || !target || !w_bf16 || !params || !grad || !loss_sum)
     return fail(ESC_EINVAL, "esc_mlp_grad: NULL argument");
-  ESC_MLP_CK(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem::total));
-  mlp_grad_kernel<<<grid_for(batch, 1), kGradThreads, GradSmem::total, static_cast<cudaStream_t>(stream)>>>(
+  int grid = 0;
+  ESC_MLP_CK(grid_for(batch, 1, &grid));
+  mlp_grad_kernel<<<grid, kGradThreads, GradSmem::total, static_cast<cudaStream_t>(stream)>>>(
       x_bf16, target, batch, w_bf16, params, grad, loss_sum);
   ESC_MLP_CK(cudaGetLastError());
   clear_error();

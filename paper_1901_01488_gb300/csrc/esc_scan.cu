@@ -2331,14 +2331,18 @@ esc_status esc_selectivity_batch(const esc_table *const *tables, const esc_pred 
   return ESC_OK;
 }
 
-esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc_pred *const *preds, int32_t n,
-                                       const esc_rows *rows, uint64_t *dev_counts, uint64_t *dev_done_ns,
-                                       void *stream) {
-  ESC_RANGE("esc_selectivity_batch_async");
-  if (n < 1 || !tables || !preds || !dev_counts)
-    return fail(ESC_EINVAL, "esc_selectivity_batch_async: need n >= 1 tables, predicates and dev_counts");
-  std::vector<Query> qs((size_t)n);
-  std::vector<uint32_t> cidx;
+// One scan and one write launch over n sub-queries.  The queries are laid out
+// in the memory they are copied from, pinned as a rule: the call does not wait
+// for the stream's earlier work (a pageable copy of this size did, and the
+// host's part of the next call then ran with the GPU idle).
+static esc_status run_batch_async(const esc_table *const *tables, const esc_pred *const *preds, int32_t n,
+                                  const esc_rows *rows, uint64_t *dev_counts, uint64_t *dev_done_ns, cudaStream_t st) {
+  const size_t q_span = (sizeof(Query) * (size_t)n + 4 * (size_t)n + 255) & ~(size_t)255;  // queries + constants' indices
+  const size_t left_bytes = ((size_t)n * 4 + 255) & ~(size_t)255;
+  HostStage stage(q_span + left_bytes, st);
+  Query *qs = reinterpret_cast<Query *>(stage.data());
+  uint32_t *cidx = reinterpret_cast<uint32_t *>(qs + n), ncidx = 0;
+  unsigned int *init = reinterpret_cast<unsigned int *>(stage.data() + q_span);
   uint64_t units = 0, wunits = 0, zeroed = 0, other = 0;
   esc_status s;
   for (int i = 0; i < n; ++i) {
@@ -2351,10 +2355,10 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
   }
   DeviceState *d;
   if ((s = device_state(&d)) != ESC_OK) return s;
-  layout_batch_write_units(qs.data(), n, d->sms);  // one write grid for all queries
+  layout_batch_write_units(qs, n, d->sms);  // one write grid for all queries
   for (int i = 0; i < n; ++i) {
     const bool compact = qs[i].mode == MODE_SELECT;
-    if (qs[i].is_const) cidx.push_back((uint32_t)i);
+    if (qs[i].is_const) cidx[ncidx++] = (uint32_t)i;
     qs[i].unit_base = (uint32_t)units;
     qs[i].wunit_base = (uint32_t)wunits;
     units += qs[i].nunits;
@@ -2365,23 +2369,19 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
     }
     if (units >= (1ull << 31)) return fail(ESC_EINVAL, "esc_selectivity_batch_async: too many work units");
   }
-  // device block: queries | zeroed: header, counts, done, countdowns, unit words | bitmaps, group data
-  const size_t q_span = (sizeof(Query) * (size_t)n + 4 * (size_t)n + 255) & ~(size_t)255;  // queries + cidx
+  // device block: queries, countdowns | zeroed: header, counts, done, unit words | bitmaps
   const size_t cnt_bytes = ((size_t)n * 8 + 255) & ~(size_t)255;
-  const size_t left_bytes = ((size_t)n * 4 + 255) & ~(size_t)255;
-  const size_t zbytes = 256 + 2 * cnt_bytes + left_bytes + (size_t)zeroed;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const size_t zbytes = 256 + 2 * cnt_bytes + (size_t)zeroed;
   void *mem = nullptr;
-  if ((s = alloc_async(&mem, q_span + zbytes + (size_t)other, st)) != ESC_OK) return s;
+  if ((s = alloc_async(&mem, q_span + left_bytes + zbytes + (size_t)other, st)) != ESC_OK) return s;
   uint8_t *base = static_cast<uint8_t *>(mem);
-  uint8_t *z = base + q_span;
+  uint8_t *z = base + q_span + left_bytes;
   unsigned long long *counts = reinterpret_cast<unsigned long long *>(z + 256);
   unsigned long long *done = reinterpret_cast<unsigned long long *>(z + 256 + cnt_bytes);
-  unsigned int *left = reinterpret_cast<unsigned int *>(z + 256 + 2 * cnt_bytes);
-  uint8_t *zp = z + 256 + 2 * cnt_bytes + left_bytes;
+  unsigned int *left = reinterpret_cast<unsigned int *>(base + q_span);
+  uint8_t *zp = z + 256 + 2 * cnt_bytes;
   uint8_t *op = z + zbytes;
-  std::vector<unsigned int> init((size_t)n);
-  const int shape = launch_shape(qs.data(), n);
+  const int shape = launch_shape(qs, n);
   for (int i = 0; i < n; ++i) {
     qs[i].count = &counts[i];
     qs[i].done_ns = dev_done_ns ? &done[i] : nullptr;
@@ -2399,11 +2399,7 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
   }
   uint32_t *dev_cidx = reinterpret_cast<uint32_t *>(base + sizeof(Query) * (size_t)n);
   cudaError_t e = cudaMemsetAsync(z, 0, zbytes, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(base, qs.data(), sizeof(Query) * (size_t)n, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !cidx.empty())
-    e = cudaMemcpyAsync(dev_cidx, cidx.data(), 4 * cidx.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && dev_done_ns)
-    e = cudaMemcpyAsync(left, init.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = stage.copy_to(base);
   if (e != cudaSuccess) {
     cudaFreeAsync(mem, st);
     return fail(ESC_ECUDA, std::string("esc_selectivity_batch_async: ") + cudaGetErrorString(e));
@@ -2414,7 +2410,7 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
   L.nq = n;
   L.total_units = (uint32_t)units;
   L.hdr = reinterpret_cast<ScratchHdr *>(z);
-  s = cidx.empty() ? ESC_OK : launch_const_batch(L.queries, dev_cidx, (uint32_t)cidx.size(), st);
+  s = ncidx == 0 ? ESC_OK : launch_const_batch(L.queries, dev_cidx, ncidx, st);
   if (s == ESC_OK) s = launch_scan(L, shape, st);
   if (s == ESC_OK) s = launch_write(L, (uint32_t)wunits, st);
   if (s == ESC_OK) {
@@ -2426,6 +2422,19 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
   cudaFreeAsync(mem, st);
   if (s == ESC_OK) clear_error();
   return s;
+}
+
+esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc_pred *const *preds, int32_t n,
+                                       const esc_rows *rows, uint64_t *dev_counts, uint64_t *dev_done_ns,
+                                       void *stream) {
+  ESC_RANGE("esc_selectivity_batch_async");
+  if (n < 1 || !tables || !preds || !dev_counts)
+    return fail(ESC_EINVAL, "esc_selectivity_batch_async: need n >= 1 tables, predicates and dev_counts");
+  try {
+    return run_batch_async(tables, preds, n, rows, dev_counts, dev_done_ns, static_cast<cudaStream_t>(stream));
+  } catch (const std::bad_alloc &) {
+    return fail(ESC_ENOMEM, "esc_selectivity_batch_async: out of host memory");
+  }
 }
 
 // Whether n predicates over `rows` rows are counted by table lookup.  It costs

@@ -117,7 +117,10 @@ def _check(status: int, where: str, ok=(ESC_OK,)) -> int:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        # the current stream's handle, without the Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
