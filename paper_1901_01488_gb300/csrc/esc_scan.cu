@@ -423,8 +423,15 @@ struct Launch {
   // which the block clears); null: none
   unsigned long long *count_out;
   HostResult *result;
-  unsigned long long seq;   // for result
-  uint32_t pad[2];
+  unsigned long long seq;     // for result: the report's last word
+  // blocks of the write kernel that are done (zeroed scratch); when set, the
+  // write kernel's last block writes seq, else the scan's
+  unsigned int *write_done;
+  // a batch's later wave: it shares nothing with the launch before it, starts
+  // while that one still runs, and waits for its end only before its own (so
+  // that what follows on the stream follows both)
+  uint32_t wait_last;
+  uint32_t pad[3];
   Query q0;
 };
 
@@ -539,6 +546,9 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
     copy_query(reinterpret_cast<uint8_t *>(qslot), L.q0, threadIdx.x - 32, 32 * NC);
   }
   __syncthreads();
+  // the kernel that clears the scratch (launch_clear) may still be running;
+  // all that was on the stream before it is done
+  if (!L.wait_last) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
@@ -636,6 +646,7 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
         }
       }
     }
+    if (L.wait_last) asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
 
@@ -777,7 +788,7 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
           *hdr = ScratchHdr{};
           *L.q0.count = 0;
           __threadfence_system();   // the slot is clear before the host can know
-          *(volatile unsigned long long *)&L.result->seq = L.seq;
+          if (!L.write_done) *(volatile unsigned long long *)&L.result->seq = L.seq;
         }
       }
     }
@@ -998,6 +1009,22 @@ __device__ __forceinline__ void lookback_load(const unsigned long long *st, cons
   }
 }
 
+// One block of the write kernel is done (thread 0, after a barrier if others
+// have stored): the last one reports to the host where the call waits for that.
+__device__ __forceinline__ void write_block_done(const Launch &L) {
+  if (!L.write_done) return;
+  __threadfence();
+  if (atomicAdd(L.write_done, 1u) == gridDim.x - 1u) {
+    __threadfence_system();
+    *(volatile unsigned long long *)&L.result->seq = L.seq;
+  }
+}
+
+// SINGLE: one sub-query, L.q0.  The launch starts as the scan's blocks end
+// (programmatic stream serialization) and waits here for the last of them.  In
+// a batch the next wave's scan is let in when the last block has started: it
+// takes the SMs that this launch's long blocks leave.
+template <bool SINGLE>
 __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel(const __grid_constant__ Launch L) {
   extern __shared__ __align__(16) uint8_t wsmem[];
   __shared__ GatherInfo G;
@@ -1008,9 +1035,12 @@ __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   WriteWarpSmem &W = reinterpret_cast<WriteWarpSmem *>(wsmem)[warp];
-  if (threadIdx.x == 0) s_q = block_query(L, [](const Query *q) { return q->wunit_base; });
-  __syncthreads();
-  const Query *Q = query_ptr(L, s_q);
+  if constexpr (!SINGLE) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (threadIdx.x == 0) s_q = block_query(L, [](const Query *q) { return q->wunit_base; });
+    __syncthreads();
+  }
+  const Query *Q = SINGLE ? &L.q0 : &L.queries[s_q];
   if (warp == 1) {
     const int np = Q->nproj;
     if (lane == 0) {
@@ -1027,7 +1057,7 @@ __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel
       G.out_proj[lane] = Q->out_proj[lane];
     }
   }
-  const uint32_t u = blockIdx.x - Q->wunit_base;
+  const uint32_t u = SINGLE ? blockIdx.x : blockIdx.x - Q->wunit_base;
   if (!ESC_INB(L.hdr, u < Q->nwunits, 20, u)) return;  // uniform: the whole block
   const uint32_t urows = Q->wunit_groups * kGroup;
   const uint32_t urow0 = u * urows;
@@ -1044,6 +1074,7 @@ __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel
   // wrote all 8 words of every group) and the first look-back window.
   const unsigned long long *tot = Q->unit_total;
   unsigned long long *st = Q->unit_status;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const unsigned long long utot = __ldcg(&tot[u]);
   uint4 wlo = make_uint4(0, 0, 0, 0), whi = wlo;
   if (valid && ESC_INB(L.hdr, grp_l < (uint64_t)Q->ntiles * Q->gmax, 21, grp_l)) {
@@ -1056,6 +1087,7 @@ __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel
   lookback_load(st, tot, idx, lw, lt);
   if (utot == 0) {
     // no qualifying row in this unit: nothing to write, nothing to publish
+    if (SINGLE && threadIdx.x == 0) write_block_done(L);
     if (Q->done_ns && threadIdx.x == 0) {
       __threadfence();
       if (atomicSub(Q->tiles_left, 1u) == 1u) *Q->done_ns = globaltimer();
@@ -1172,6 +1204,12 @@ __global__ void __launch_bounds__(kWriteThreads, kWriteBlocksPerSm) write_kernel
         flush_sparse(G, ent, min(stot - win, kStageEntries), row_ref, pos_ref, lane, L.hdr);
         __syncwarp();
       }
+    }
+  }
+  if constexpr (SINGLE) {
+    if (L.write_done) {
+      __syncthreads();
+      if (threadIdx.x == 0) write_block_done(L);
     }
   }
   // per-query completion time: the query's last write block
@@ -1402,6 +1440,14 @@ __global__ void __launch_bounds__(256) const_batch_kernel(const Query *queries, 
   }
 }
 
+// Clears a single sub-query's scratch.  The scan is let in at once: it stages
+// its query meanwhile and waits for this grid before it touches the scratch.
+__global__ void __launch_bounds__(256) clear_kernel(uint4 *p, uint64_t n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+    p[i] = make_uint4(0, 0, 0, 0);
+}
+
 // A kernel whose only job is a bounded wait on a flag that nothing sets.
 __global__ void wait_selftest_kernel(const unsigned *flag, ScratchHdr *hdr, uint64_t limit_ns) {
   const uint64_t t0 = globaltimer();
@@ -1443,21 +1489,32 @@ struct ScanInstance {
   static constexpr ScanShape sh = kScanShapes[S];
   static constexpr int threads = 32 * (sh.consumers + 1);
   static const void *fn() { return reinterpret_cast<const void *>(scan_kernel<sh.consumers, sh.udf, sh.groups>); }
-  static void launch(uint32_t grid, const Launch &L, cudaStream_t st) {
-    scan_kernel<sh.consumers, sh.udf, sh.groups><<<grid, threads, smem_bytes(), st>>>(L);
-  }
 };
+
+// Launches a kernel; `early`: it may start while the kernel before it on the
+// stream still runs (it waits for that one's end itself).
+cudaError_t launch_kernel(const void *fn, uint32_t grid, uint32_t threads, size_t smem, const Launch &L, bool early,
+                          cudaStream_t st) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  void *args[] = {const_cast<Launch *>(&L)};
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
 static_assert(kNumScanShapes == 5, "one ScanInstance per shape below");
 
 // Launches the scan kernel instance of block shape `shape`.
-void launch_scan_shape(int shape, uint32_t grid, const Launch &L, cudaStream_t st) {
-  switch (shape) {
-    case 0: ScanInstance<0>::launch(grid, L, st); break;
-    case 1: ScanInstance<1>::launch(grid, L, st); break;
-    case 2: ScanInstance<2>::launch(grid, L, st); break;
-    case 3: ScanInstance<3>::launch(grid, L, st); break;
-    default: ScanInstance<4>::launch(grid, L, st); break;
-  }
+cudaError_t launch_scan_shape(int shape, uint32_t grid, const Launch &L, bool early, cudaStream_t st) {
+  const void *fns[kNumScanShapes] = {ScanInstance<0>::fn(), ScanInstance<1>::fn(), ScanInstance<2>::fn(),
+                                     ScanInstance<3>::fn(), ScanInstance<4>::fn()};
+  return launch_kernel(fns[shape], grid, 32u * (kScanShapes[shape].consumers + 1), smem_bytes(), L, early, st);
 }
 
 // Kernel attributes (dynamic shared memory) of every kernel of this file,
@@ -1475,7 +1532,8 @@ esc_status configure_kernels(int *blocks_per_sm) {
     b = std::min(b, k);
   }
   if (b < 1) return fail(ESC_ECUDA, "a scan kernel instance does not fit on an SM");
-  ESC_CK(cudaFuncSetAttribute(write_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWriteSmem));
+  ESC_CK(cudaFuncSetAttribute(write_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWriteSmem));
+  ESC_CK(cudaFuncSetAttribute(write_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWriteSmem));
   ESC_CK(cudaFuncSetAttribute(shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SharedSmem::total));
   *blocks_per_sm = b;
   return ESC_OK;
@@ -1802,24 +1860,36 @@ esc_status alloc_async(void **p, size_t bytes, cudaStream_t st) {
   return ESC_OK;
 }
 
+// Clears `bytes` (a multiple of 16) of a single sub-query's scratch; the scan
+// that follows is launched early.  A memset in its place cost a count of a
+// small table about 2 us (it cannot overlap the scan's start).
+esc_status launch_clear(void *p, size_t bytes, cudaStream_t st) {
+  const uint64_t n = bytes / 16;
+  clear_kernel<<<(uint32_t)std::min<uint64_t>(64, (n + 255) / 256), 256, 0, st>>>(static_cast<uint4 *>(p), n);
+  ESC_CK(cudaGetLastError());
+  return ESC_OK;
+}
+
 // shape: the block shape (kScanShapes) of the instance that runs the launch.
-esc_status launch_scan(const Launch &L, int shape, cudaStream_t st) {
+// early: launch_clear comes right before it on the stream.
+esc_status launch_scan(const Launch &L, int shape, cudaStream_t st, bool early = false) {
   DeviceState *d;
   esc_status s = device_state(&d);
   if (s != ESC_OK) return s;
   if (L.total_units == 0) return ESC_OK;
   const uint32_t cap = (uint32_t)(d->sms * d->blocks_per_sm);
   const uint32_t grid = std::min<uint32_t>(cap, L.total_units);
-  launch_scan_shape(shape, grid, L, st);
-  ESC_CK(cudaGetLastError());
+  ESC_CK(launch_scan_shape(shape, grid, L, early, st));
   return ESC_OK;
 }
 
 // Second pass of compaction: the write kernel, one block per compaction unit.
 esc_status launch_write(const Launch &L, uint32_t unit_blocks, cudaStream_t st) {
   if (unit_blocks == 0) return ESC_OK;
-  write_kernel<<<unit_blocks, kWriteThreads, kWriteSmem, st>>>(L);
-  ESC_CK(cudaGetLastError());
+  const bool single = L.queries == nullptr;
+  ESC_CK(launch_kernel(single ? reinterpret_cast<const void *>(write_kernel<true>)
+                              : reinterpret_cast<const void *>(write_kernel<false>),
+                       unit_blocks, kWriteThreads, kWriteSmem, L, true, st));
   return ESC_OK;
 }
 
@@ -1899,11 +1969,13 @@ esc_status run_single(const esc_table *t, const esc_pred *p, esc_rows *rows, int
   uint32_t cval = 0;
   const bool constant = program_constant(L.q0, &cval);
   const bool direct = dev_count && !constant && L.total_units > 0;
-  cudaError_t e = cudaMemsetAsync(mem, 0, head + zeroed, st);
-  if (e == cudaSuccess && dev_count && !direct) e = cudaMemsetAsync(dev_count, 0, sizeof(unsigned long long), st);
-  if (e != cudaSuccess) {
+  cudaError_t e = cudaSuccess;
+  if (dev_count && !direct) e = cudaMemsetAsync(dev_count, 0, sizeof(unsigned long long), st);
+  s = e == cudaSuccess ? launch_clear(mem, head + zeroed, st)
+                       : fail(ESC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+  if (s != ESC_OK) {
     cudaFreeAsync(mem, st);
-    return fail(ESC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+    return s;
   }
   uint8_t *base = static_cast<uint8_t *>(mem);
   SingleScratch *sc = static_cast<SingleScratch *>(mem);
@@ -1914,7 +1986,7 @@ esc_status run_single(const esc_table *t, const esc_pred *p, esc_rows *rows, int
   if (constant) {
     s = launch_const(L, cval, st);
   } else {
-    s = launch_scan(L, query_shape(L.q0, p->tuning), st);
+    s = launch_scan(L, query_shape(L.q0, p->tuning), st, true);
     if (s == ESC_OK && mode == MODE_SELECT) s = launch_write(L, L.q0.nwunits, st);
   }
   if (s != ESC_OK) {
@@ -1956,29 +2028,27 @@ esc_status run_sync(const esc_table *t, const esc_pred *p, esc_rows *rows, int m
   L.result = slot.host_dev;
   L.seq = slot.seq;
   void *mem = nullptr;
-  cudaError_t e = cudaSuccess;
-  if (mode == MODE_SELECT) {   // unit totals and look-back words (zeroed), selection bitmap
-    const size_t zeroed = select_zeroed_bytes(L.q0);
+  if (mode == MODE_SELECT) {   // write blocks done, unit totals, look-back words (zeroed), selection bitmap
+    const size_t zeroed = 256 + select_zeroed_bytes(L.q0);
     if ((s = alloc_async(&mem, zeroed + select_other_bytes(L.q0), st)) != ESC_OK) {
       give_slot(slot);
       return s;
     }
-    e = cudaMemsetAsync(mem, 0, zeroed, st);
-    select_bind(L.q0, static_cast<uint8_t *>(mem), static_cast<uint8_t *>(mem) + zeroed);
-    if (e != cudaSuccess) {
+    L.write_done = static_cast<unsigned int *>(mem);
+    select_bind(L.q0, static_cast<uint8_t *>(mem) + 256, static_cast<uint8_t *>(mem) + zeroed);
+    if ((s = launch_clear(mem, zeroed, st)) != ESC_OK) {
       cudaFreeAsync(mem, st);
       give_slot(slot);
-      return fail(ESC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+      return s;
     }
   }
-  s = launch_scan(L, query_shape(L.q0, p->tuning), st);
+  s = launch_scan(L, query_shape(L.q0, p->tuning), st, mem != nullptr);
   if (s == ESC_OK && mode == MODE_SELECT) s = launch_write(L, L.q0.nwunits, st);
   if (mem) cudaFreeAsync(mem, st);
   // (after a failure the slot stays taken: its launch may still be running)
   if (s != ESC_OK) return s;
-  // the scan reports its count; rows are written after it
-  if (mode == MODE_SELECT || !poll_slot(slot)) {
-    e = cudaStreamSynchronize(st);
+  if (!poll_slot(slot)) {
+    const cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("sub-query: ") + cudaGetErrorString(e));
   }
   ScratchHdr h{};
@@ -2245,7 +2315,9 @@ esc_status batch_prepare(const esc_table *const *tables, const esc_pred *const *
       L.nq = wend[w] - k0;
       L.total_units = w_units[w];
       L.hdr = reinterpret_cast<ScratchHdr *>(b->scratch + 256 * (size_t)w);
-      ls = launch_scan(L, w_shape[w], cs);
+      // (the wave before ended with a scan or write launch; the first follows a copy)
+      L.wait_last = w > 0 && (w_units[w - 1] > 0 || w_wunits[w - 1] > 0) ? 1u : 0u;
+      ls = launch_scan(L, w_shape[w], cs, L.wait_last != 0);
       if (ls == ESC_OK) ls = launch_write(L, w_wunits[w], cs);
     }
     e = cudaStreamEndCapture(cs, &b->graph);
@@ -2717,12 +2789,8 @@ extern "C" esc_status esc_selectivity_noalloc(const esc_table *t, const esc_pred
     ESC_CK(cudaGetLastError());
   } else if (L.total_units > 0) {
     const uint32_t grid = std::min<uint32_t>((uint32_t)(d->sms * d->blocks_per_sm), L.total_units);
-    launch_scan_shape(query_shape(q, p->tuning), grid, L, st);
-    ESC_CK(cudaGetLastError());
-    if (mode == MODE_SELECT) {
-      write_kernel<<<q.nwunits, kWriteThreads, kWriteSmem, st>>>(L);
-      ESC_CK(cudaGetLastError());
-    }
+    ESC_CK(launch_scan_shape(query_shape(q, p->tuning), grid, L, false, st));
+    if (mode == MODE_SELECT && (s = launch_write(L, q.nwunits, st)) != ESC_OK) return s;
   }
   NoAllocHead back;
   ESC_CK(cudaMemcpyAsync(&back, h, sizeof back, cudaMemcpyDeviceToHost, st));

@@ -67,13 +67,19 @@ def test_calls_around_a_capture():
     p = [esc.Predicate(t, x) for x in TEXTS]
     want = [esc.count(t, x) for x in p]
     out = torch.zeros(len(p), dtype=torch.int64, device="cuda")
+    rows = [x.alloc_rows(c + 1) for x, c in zip(p, want)]
+    ids = [esc.select(t, x)[1].clone() for x in p]
     g = torch.cuda.CUDAGraph()
     side = torch.cuda.Stream()
     with torch.cuda.graph(g, capture_error_mode="thread_local"):
         for k, x in enumerate(p):
-            esc.esc_selectivity_async(t.handle, x.handle, out[k:k + 1])
+            esc.esc_selectivity_async(t.handle, x.handle, out[k:k + 1], rows[k] if k % 2 else None)
         assert esc.count(t, p[0], side) == want[0]
     for _ in range(2):
         out.zero_()
+        for r in rows:
+            r[1].fill_(-1)
         g.replay()
         assert out.tolist() == want
+        for k in range(1, len(p), 2):
+            assert torch.equal(rows[k][1][:want[k]], ids[k]) and rows[k][1][want[k]].item() == -1
