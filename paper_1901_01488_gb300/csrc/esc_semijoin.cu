@@ -1,22 +1,29 @@
 // Exact semi-join cardinalities over dense keys: the COUNT(*) foreign-key
 // join queries of the paper's overhead experiments (Sec. 3.1: lineitem joined
 // with a filtered orders / part / supplier table) generalised to a star
-// schema.  One pass over the fact table's foreign-key columns:
-//   m(i) = sum_d [0 <= fk_d[i] < D_d and bitmap_d bit fk_d[i]] << d,
-//   h[v] = |{ i : m(i) = v }|          (2^ndims bins)
-// and on the host, for every dimension subset S,
-//   count(S) = sum over v that contain S of h[v]   (superset sum).
+// schema.  One pass over the fact table's foreign-key columns: a row matches in
+// dimension d when 0 <= fk_d < D_d and bit fk_d of bitmap_d is set, and for
+// every dimension subset S,
+//   count(S) = |{ rows that match in all of S }|.
 //
-// Kernel shape: persistent grid of one block of 512 threads per SM (shared
-// memory sized to the bitmaps it holds, the rest of the SM's on-chip memory
-// left to L1; up to 128 registers a thread); each thread streams 8 rows per
-// step with 16-byte non-allocating loads of every FK column (4 rows per
-// load).  The kernel is specialised on how many bitmaps sit in shared memory
-// (dimensions are ordered smallest bitmap first, so the shared ones come
-// first): each probe is then a fixed sequence -- clamp the word index, load,
-// shift, mask with the bounds test.  The 16 bins are 8-bit
-// counters in two 64-bit registers, added into shared per-block bins (warp
-// reductions) before they can overflow.
+// Kernel shape: persistent grid of one block per SM (shared memory sized to the
+// bitmaps it holds, the rest of the SM's on-chip memory left to L1); a warp
+// streams 256 rows per step, 512 consecutive bytes per non-allocating load of a
+// foreign-key column, 8 rows a lane.  The kernel is specialised on how many
+// bitmaps sit in shared memory (dimensions are ordered smallest bitmap first,
+// so the shared ones come first): each probe is then a fixed sequence -- clamp
+// the word index, load, two funnel shifts that append the key's bit to the
+// lane's bits of that dimension.  Every 32 rows the subsets' bits are ANDed and
+// counted (15 popcounts for four dimensions).
+// What bounds it: L1's data pipe (it was 92 % busy with 32 bytes per lane and
+// load, which read every sector twice) for large bitmaps, HBM next.  Measured
+// at 120M rows, before (each lane 8 consecutive rows, 16 byte counters per
+// thread, 512 threads) and now: dimensions of 2M, 200K, 30K and 2,556 rows 373
+// -> 320 us a call, one of 2M 200 -> 149, 900K and 30K 209 -> 162, 8M and 2M
+// 714 -> 712.  By threads per block: four dimensions 512 / 640 / 768 / 1024:
+// 360 / 329 / 320 / 328; one: 183 / 161 / 151 / 149.  Holding part of a large
+// bitmap in shared memory did not help (a gather there costs what one in L1
+// does).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,10 +32,13 @@
 #include <string>
 
 #include "esc_internal.h"
+#include "esc_ptx.cuh"
 
 namespace esc {
 
-constexpr int kSjThreads = 512;
+constexpr uint32_t kSjWarpRows = 256;   // rows a warp takes per step: 8 per lane
+// Threads of a block (one per SM; measured above): more where few dimensions leave registers.
+constexpr uint32_t sj_threads(int ndims) { return ndims <= 2 ? 1024 : 768; }
 constexpr int kSjMaxDims = 4;
 constexpr uint32_t kSjSmemBitmapBytes = 96 * 1024;  // shared copies of the smaller bitmaps
 
@@ -40,7 +50,7 @@ struct SjParams {
   uint32_t words[kSjMaxDims];
   int32_t ndims;
   uint32_t nrows;
-  unsigned long long *hist;            // 16 bins, zeroed
+  unsigned long long *hist;            // 16 subset counts, zeroed
   ScratchHdr *hdr;                     // launch header (zeroed): blocks done, the checked build's findings
   HostResult *result;                  // hist and hdr are a call slot: the last block reports here and clears them
   unsigned long long seq;              // for result
@@ -55,63 +65,65 @@ __device__ __forceinline__ int4 ld_stream(const int32_t *p) {
   return v;
 }
 
-// Bit `key` of a bitmap of `rows` bits, 0 when key is out of range (negative
-// keys wrap to large unsigned values).  A shared-memory copy ends with a zero
-// word at index `wlast` and has the bits past `rows` cleared, so clamping the
-// word index is the whole bounds test there; a bitmap read in place is
-// tested explicitly.
-__device__ __forceinline__ uint32_t test_bit(const uint32_t *bm, uint32_t key, uint32_t rows, uint32_t wlast,
-                                             bool shared) {
-  if (shared) return (bm[min(key >> 5, wlast)] >> (key & 31u)) & 1u;
+// The word that holds bit `key` of a bitmap of `rows` bits; a word whose bit
+// is 0 when key is out of range (negative keys wrap to large unsigned values).
+// A shared-memory copy ends with a zero word at index `wlast` and has the bits
+// past `rows` cleared, so clamping the word index is the whole bounds test
+// there; a bitmap read in place is tested explicitly.
+__device__ __forceinline__ uint32_t probe_word(const uint32_t *bm, uint32_t key, uint32_t rows, uint32_t wlast,
+                                               bool shared) {
+  if (shared) return bm[min(key >> 5, wlast)];
   const uint32_t w = __ldg(&bm[min(key >> 5, wlast)]);
-  return key < rows ? (w >> (key & 31u)) & 1u : 0u;
+  return key < rows ? w : 0u;
 }
 
 // The same, in the checked build: the word index is tested against the
 // bitmap's words (in shared memory: its copy and the zero word).
-__device__ __forceinline__ uint32_t test_bit_checked(const uint32_t *bm, uint32_t key, uint32_t rows, uint32_t wlast,
-                                                     bool shared, uint32_t words, ScratchHdr *hdr) {
+__device__ __forceinline__ uint32_t probe_word_checked(const uint32_t *bm, uint32_t key, uint32_t rows, uint32_t wlast,
+                                                       bool shared, uint32_t words, ScratchHdr *hdr) {
   const uint32_t wi = min(key >> 5, wlast);
   if (!ESC_INB(hdr, wi < (shared ? words + 1 : words), 32, wi)) return 0u;
-  return test_bit(bm, key, rows, wlast, shared);
+  return probe_word(bm, key, rows, wlast, shared);
 }
 
-__device__ __forceinline__ void bump(uint64_t &lo, uint64_t &hi, uint32_t m) {
-  const uint64_t inc = 1ull << (8u * (m & 7u));
-  if (m & 8u) hi += inc; else lo += inc;
-}
+// A thread's rows as bits: bits[d] collects the rows' matches in dimension d,
+// 32 rows at most; count() adds, for every subset of the dimensions, the rows
+// that match all of it.
+template <int ND, int NS>
+struct RowBits {
+  uint32_t bits[ND] = {};
+  uint32_t n[1 << ND] = {};   // by subset (0: unused)
 
-// Adds this warp's byte counters into the block's bins.
-__device__ __forceinline__ void flush(uint64_t &lo, uint64_t &hi, unsigned int *bins) {
+  __device__ __forceinline__ void row(const SjParams &P, const uint32_t *const (&bm)[ND], const uint32_t (&wmax)[ND],
+                                      const int32_t (&k)[ND]) {
 #pragma unroll
-  for (int v = 0; v < 8; ++v) {
-    const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)((lo >> (8 * v)) & 0xffu));
-    const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)((hi >> (8 * v)) & 0xffu));
-    if ((threadIdx.x & 31) == 0) {
-      if (a) atomicAdd(&bins[v], a);
-      if (b) atomicAdd(&bins[v + 8], b);
+    for (int d = 0; d < ND; ++d) {
+      const uint32_t key = (uint32_t)k[d];
+#ifdef ESC_CHECKED
+      const uint32_t w = probe_word_checked(bm[d], key, P.dim_rows[d], wmax[d], d < NS, P.words[d], P.hdr);
+#else
+      const uint32_t w = probe_word(bm[d], key, P.dim_rows[d], wmax[d], d < NS);
+#endif
+      // the key's bit to the top of the word, and from there into the collected ones
+      bits[d] = __funnelshift_l(__funnelshift_l(w, w, ~key), bits[d], 1);
     }
   }
-  lo = hi = 0;
-}
-
-template <int ND, int NS>
-__device__ __forceinline__ uint32_t probe_row(const SjParams &P, const uint32_t *const (&bm)[ND],
-                                              const uint32_t (&wmax)[ND], const int32_t (&k)[ND]) {
-  uint32_t m = 0;
+  __device__ __forceinline__ void count() {
+    uint32_t s[1 << ND];
 #pragma unroll
-  for (int d = 0; d < ND; ++d) {
-#ifdef ESC_CHECKED
-    m |= test_bit_checked(bm[d], (uint32_t)k[d], P.dim_rows[d], wmax[d], d < NS, P.words[d], P.hdr) << d;
-#else
-    m |= test_bit(bm[d], (uint32_t)k[d], P.dim_rows[d], wmax[d], d < NS) << d;
-#endif
+    for (int v = 1; v < (1 << ND); ++v) {
+      const int low = v & -v, rest = v ^ low;   // the subset without its first dimension
+      const int d = low == 1 ? 0 : low == 2 ? 1 : low == 4 ? 2 : 3;
+      s[v] = rest ? s[rest] & bits[d] : bits[d];
+      n[v] += __popc(s[v]);
+    }
+#pragma unroll
+    for (int d = 0; d < ND; ++d) bits[d] = 0;
   }
-  return m;
-}
+};
 
 template <int ND, int NS>
-__global__ void __launch_bounds__(kSjThreads, 1) semijoin_kernel(const __grid_constant__ SjParams P) {
+__global__ void __launch_bounds__(sj_threads(ND), 1) semijoin_kernel(const __grid_constant__ SjParams P) {
   extern __shared__ __align__(16) uint32_t sbm[];
   __shared__ unsigned int bins[16];
 #pragma unroll
@@ -134,52 +146,55 @@ __global__ void __launch_bounds__(kSjThreads, 1) semijoin_kernel(const __grid_co
     wmax[d] = d < NS ? P.words[d] : P.words[d] - 1u;  // shared: the zero word; global: words >= 1
   }
 
-  uint64_t lo = 0, hi = 0;
-  uint32_t pending = 0;
-  const uint32_t nchunks = P.nrows / 8u;  // 8 rows per thread step
-  const uint32_t stride = gridDim.x * blockDim.x;
-  // warp-uniform trip count (the flush is warp-collective); lanes past the end idle
-  for (uint32_t wb = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); wb < nchunks; wb += stride) {
-    const uint32_t ch = wb + (threadIdx.x & 31u);
-    if (ch < nchunks && ESC_INB(P.hdr, (uint64_t)ch * 8 + 8 <= P.nrows, 30, ch)) {
-    int4 v[ND][2];
+  RowBits<ND, NS> R;
+  // A warp's loads are 512 consecutive bytes: lane l takes rows 4l .. 4l + 3 of
+  // either half of the warp's 256 rows.
+  const uint32_t nchunks = P.nrows / kSjWarpRows;
+  const uint32_t stride = gridDim.x * (blockDim.x / 32);
+  uint32_t steps = 0;
+  for (uint32_t ch = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); ch < nchunks; ch += stride) {
+    const uint32_t r0 = ch * kSjWarpRows + 4u * (threadIdx.x & 31u);
+    if (ESC_INB(P.hdr, (uint64_t)r0 + 132 <= P.nrows, 30, r0)) {
+      int4 v[ND][2];
 #pragma unroll
-    for (int d = 0; d < ND; ++d)
+      for (int d = 0; d < ND; ++d)
 #pragma unroll
-      for (int q = 0; q < 2; ++q) v[d][q] = ld_stream(P.fk[d] + (size_t)ch * 8 + 4 * q);
+        for (int q = 0; q < 2; ++q) v[d][q] = ld_stream(P.fk[d] + (size_t)r0 + 128 * q);
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      int32_t k0[ND], k1[ND], k2[ND], k3[ND];
+      for (int q = 0; q < 2; ++q) {
+        int32_t k0[ND], k1[ND], k2[ND], k3[ND];
 #pragma unroll
-      for (int d = 0; d < ND; ++d) {
-        k0[d] = v[d][q].x;
-        k1[d] = v[d][q].y;
-        k2[d] = v[d][q].z;
-        k3[d] = v[d][q].w;
+        for (int d = 0; d < ND; ++d) {
+          k0[d] = v[d][q].x;
+          k1[d] = v[d][q].y;
+          k2[d] = v[d][q].z;
+          k3[d] = v[d][q].w;
+        }
+        R.row(P, bm, wmax, k0);
+        R.row(P, bm, wmax, k1);
+        R.row(P, bm, wmax, k2);
+        R.row(P, bm, wmax, k3);
       }
-      bump(lo, hi, probe_row<ND, NS>(P, bm, wmax, k0));
-      bump(lo, hi, probe_row<ND, NS>(P, bm, wmax, k1));
-      bump(lo, hi, probe_row<ND, NS>(P, bm, wmax, k2));
-      bump(lo, hi, probe_row<ND, NS>(P, bm, wmax, k3));
     }
-    }
-    pending += 8;
-    if (pending >= 248) {  // 8-bit counters: flush before any can pass 255
-      flush(lo, hi, bins);
-      pending = 0;
-    }
+    if ((++steps & 3u) == 0) R.count();   // 32 rows
   }
-  // ragged tail: rows nchunks*8 .. nrows-1, one per thread of block 0
+  R.count();
+  // ragged tail: rows nchunks*256 .. nrows-1, one per thread of block 0
   if (blockIdx.x == 0) {
-    const uint32_t r = nchunks * 8u + threadIdx.x;
+    const uint32_t r = nchunks * kSjWarpRows + threadIdx.x;   // nrows <= 2^32 - 2^16: no overflow
     if (r < P.nrows) {
       int32_t k[ND];
 #pragma unroll
       for (int d = 0; d < ND; ++d) k[d] = P.fk[d][r];
-      bump(lo, hi, probe_row<ND, NS>(P, bm, wmax, k));
+      R.row(P, bm, wmax, k);
     }
+    R.count();
   }
-  flush(lo, hi, bins);
+#pragma unroll
+  for (int v = 1; v < (1 << ND); ++v) {
+    const uint32_t t = __reduce_add_sync(0xffffffffu, R.n[v]);
+    if ((threadIdx.x & 31) == 0 && t) atomicAdd(&bins[v], t);
+  }
   __syncthreads();
   if (threadIdx.x < 16 && bins[threadIdx.x]) atomicAdd(&P.hist[threadIdx.x], (unsigned long long)bins[threadIdx.x]);
   if (P.result && threadIdx.x < 32) {
@@ -205,7 +220,7 @@ __global__ void __launch_bounds__(kSjThreads, 1) semijoin_kernel(const __grid_co
 }
 
 template <int ND, int NS>
-cudaError_t launch_semijoin(const SjParams &P, size_t smem, int grid, cudaStream_t st) {
+cudaError_t launch_semijoin(const SjParams &P, size_t smem, int sms, cudaStream_t st) {
   static std::once_flag once[64];
   static cudaError_t attr[64];
   int dev = 0;
@@ -220,18 +235,21 @@ cudaError_t launch_semijoin(const SjParams &P, size_t smem, int grid, cudaStream
                                             (int)cudaSharedmemCarveoutMaxL1);
   });
   if (attr[dev & 63] != cudaSuccess) return attr[dev & 63];
-  semijoin_kernel<ND, NS><<<grid, kSjThreads, smem, st>>>(P);
+  constexpr uint32_t threads = sj_threads(ND);
+  const uint32_t chunks = P.nrows / kSjWarpRows;
+  const int grid = std::max(1, std::min<int>(sms, (int)((chunks + threads / 32 - 1) / (threads / 32))));
+  semijoin_kernel<ND, NS><<<grid, threads, smem, st>>>(P);
   return cudaGetLastError();
 }
 
 template <int ND>
-cudaError_t launch_nd(const SjParams &P, int ns, size_t smem, int grid, cudaStream_t st) {
+cudaError_t launch_nd(const SjParams &P, int ns, size_t smem, int sms, cudaStream_t st) {
   switch (ns) {
-    case 0: return launch_semijoin<ND, 0>(P, smem, grid, st);
-    case 1: return launch_semijoin<ND, (ND >= 1 ? 1 : 0)>(P, smem, grid, st);
-    case 2: return launch_semijoin<ND, (ND >= 2 ? 2 : 0)>(P, smem, grid, st);
-    case 3: return launch_semijoin<ND, (ND >= 3 ? 3 : 0)>(P, smem, grid, st);
-    default: return launch_semijoin<ND, ND>(P, smem, grid, st);
+    case 0: return launch_semijoin<ND, 0>(P, smem, sms, st);
+    case 1: return launch_semijoin<ND, (ND >= 1 ? 1 : 0)>(P, smem, sms, st);
+    case 2: return launch_semijoin<ND, (ND >= 2 ? 2 : 0)>(P, smem, sms, st);
+    case 3: return launch_semijoin<ND, (ND >= 3 ? 3 : 0)>(P, smem, sms, st);
+    default: return launch_semijoin<ND, ND>(P, smem, sms, st);
   }
 }
 
@@ -290,7 +308,7 @@ extern "C" esc_status esc_semijoin_counts(const esc_table *fact, const char *con
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // a call slot, or scratch from the library's device pool (memory stays
-  // reserved between calls): 16 bins, then the launch header
+  // reserved between calls): 16 counts, then the launch header
   void *mem = nullptr;
   SlotRef slot;
   const bool in_slot = take_slot(st, &slot);
@@ -315,14 +333,12 @@ extern "C" esc_status esc_semijoin_counts(const esc_table *fact, const char *con
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = (size_t)std::max<uint32_t>(smem_words, 4) * 4;
   P.smem_words = (uint32_t)(smem / 4);
-  const uint32_t chunks = P.nrows / 8u;
-  const int grid = std::max(1, std::min<int>(sms, (int)((chunks + kSjThreads - 1) / kSjThreads)));
   if (e == cudaSuccess) {
     switch (ndims) {
-      case 1: e = launch_nd<1>(P, ns, smem, grid, st); break;
-      case 2: e = launch_nd<2>(P, ns, smem, grid, st); break;
-      case 3: e = launch_nd<3>(P, ns, smem, grid, st); break;
-      default: e = launch_nd<4>(P, ns, smem, grid, st); break;
+      case 1: e = launch_nd<1>(P, ns, smem, sms, st); break;
+      case 2: e = launch_nd<2>(P, ns, smem, sms, st); break;
+      case 3: e = launch_nd<3>(P, ns, smem, sms, st); break;
+      default: e = launch_nd<4>(P, ns, smem, sms, st); break;
     }
   }
   struct {
@@ -341,19 +357,12 @@ extern "C" esc_status esc_semijoin_counts(const esc_table *fact, const char *con
     give_slot(slot);
   }
   if (back.hdr.status != 0) return device_status(back.hdr, "esc_semijoin_counts");
-  // bins are in probe order (bit i = dimension order[i]): back to the caller's bits
-  const uint32_t nsub = 1u << ndims;
-  uint64_t hc[16] = {0};
-  for (uint32_t v = 0; v < nsub; ++v) {
-    uint32_t vc = 0;
-    for (int i = 0; i < ndims; ++i) vc |= ((v >> i) & 1u) << order[i];
-    hc[vc] += h[v];
-  }
-  for (uint32_t S = 0; S < nsub; ++S) {
-    uint64_t sum = 0;
-    for (uint32_t v = 0; v < nsub; ++v)
-      if ((v & S) == S) sum += hc[v];
-    subset_counts[S] = sum;
+  // subsets are in probe order (bit i = dimension order[i]): back to the caller's bits
+  subset_counts[0] = fact->nrows;
+  for (uint32_t v = 1; v < (1u << ndims); ++v) {
+    uint32_t S = 0;
+    for (int i = 0; i < ndims; ++i) S |= ((v >> i) & 1u) << order[i];
+    subset_counts[S] = h[v];
   }
   clear_error();
   return ESC_OK;
