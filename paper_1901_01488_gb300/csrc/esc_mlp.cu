@@ -40,7 +40,8 @@ namespace esc {
 
 constexpr int kIn = 64, kH = 128;            // inputs, hidden width
 constexpr int kTileS = 128;                  // samples per tile (rows of an accumulator: one tensor-memory lane each)
-constexpr int kFwdThreads = 256, kGradThreads = 256;   // two warps per 32 lanes of tensor memory: half of the columns each
+constexpr int kFwdThreads = 256;    // two warps per 32 lanes of tensor memory: half of the columns each
+constexpr int kGradThreads = 512;   // four, a quarter of the columns each
 constexpr int kW1 = 0, kB1 = kW1 + kH * kIn, kW2 = kB1 + kH, kB2 = kW2 + kH * kH, kW3 = kB2 + kH, kB3 = kW3 + kH;
 constexpr int kParams = kB3 + 1;  // 24961
 static_assert(kParams == ESC_MLP_PARAMS, "flat parameter layout");
@@ -107,6 +108,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(addr));
 }
 __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t (&r)[16]) {
@@ -385,13 +393,15 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
 // multiplied with it, column 0 then 1 for gb1.
 // R holds z1, then dy z1, then d1, in three parts of two blocks.
 // What bounds it at 4096 samples (32 tiles on 32 SMs): the chain of products
-// and conversions of one tile and the loading of weights.  A training step
-// (two fills, this, Adam; bound by the host's launches up to 20,000 samples):
-// 4096 samples 51.7 -> 35.8 us, 20,000 162 -> 45, 65,536 417 -> 80.
+// and conversions of one tile, the loading of weights, and the fetching of
+// instructions that each block runs once (20 us here by ncu, 24 with 256
+// threads and twice the code, 43 before the tensor cores).  A training step
+// (two fills, this, Adam): 4096 samples 50.5 -> 28.6 us, 20,000 162 -> 47,
+// 65,536 417 -> 76.
 constexpr uint32_t kTgB = 384, kTm = 448, kTgW1 = 448;
 struct GradSmem {
   static constexpr uint32_t w1 = 0, w2 = kBlock, x = 3 * kBlock, e = 4 * kBlock, mask = 5 * kBlock, r = 7 * kBlock,
-                            vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * kTileS, tmem = bar + 16,
+                            vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * 4 * kTileS, tmem = bar + 16,
                             total = tmem + 16;
 };
 
@@ -415,9 +425,9 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [2]
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + GradSmem::tmem);
   uint8_t *R = sm + GradSmem::r, *E = sm + GradSmem::e, *mask = sm + GradSmem::mask;
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, half = warp >> 2, row = threadIdx.x & 127u;
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, quarter = warp >> 2, row = threadIdx.x & 127u;
   const bool vec = ((uintptr_t)x & 15u) == 0, gvec = ((uintptr_t)grad & 15u) == 0;
-  uint4 xr[4];
+  uint4 xr[2];
   load_x<kGradThreads>(x, B, (uint64_t)blockIdx.x * kTileS, vec, xr);
   if (warp == 0) tmem_alloc(slot, kTmCols);
   if (threadIdx.x == 0) {
@@ -427,13 +437,13 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   }
   load_weights<kGradThreads>(sm + GradSmem::w1, sm + GradSmem::w2, V, wbf, pf);
 #pragma unroll
-  for (uint32_t c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(chunk(E, row, 4 * half + c)) = make_uint4(0, 0, 0, 0);
+  for (uint32_t c = 0; c < 2; ++c) *reinterpret_cast<uint4 *>(chunk(E, row, 2 * quarter + c)) = make_uint4(0, 0, 0, 0);
   store_x<kGradThreads>(sm + GradSmem::x, xr);
   fence_proxy_async_smem();
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
-  const uint32_t tm = *slot, lanes = tm + ((warp & 3u) << 21);
+  const uint32_t tm = *slot, lanes = tm + ((warp & 3u) << 21), mine = lanes + 32 * quarter;   // its 32 columns of 128
   const uint64_t dw1 = sdesc(smem_addr(sm + GradSmem::w1)), dw2 = sdesc(smem_addr(sm + GradSmem::w2)),
                  dx = sdesc(smem_addr(sm + GradSmem::x)), de = sdesc(smem_addr(E)), dm = sdesc(smem_addr(mask)),
                  dr = sdesc(smem_addr(R));
@@ -452,15 +462,11 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr);
     ph0 ^= 1u;
     tc_after_sync();
-    float2 z1[32];
+    float2 z1[16], v[16];
+    load_sum32x4(mine, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float2 v[16];
-      load_sum32x4(lanes + 64 * half + 32 * h, v);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) z1[16 * h + k] = relu_bias(v[k], V.b1 + 64 * half + 32 * h + 2 * k);
-      store_split32<true>(R, 2 * half + h, row, z1 + 16 * h);
-    }
+    for (int k = 0; k < 16; ++k) z1[k] = relu_bias(v[k], V.b1 + 32 * quarter + 2 * k);
+    store_split32<true>(R, quarter, row, z1);
     fence_proxy_async_smem();
     tc_before_sync();
     __syncthreads();
@@ -472,40 +478,35 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
     ph0 ^= 1u;
     tc_after_sync();
+    // y, the mask, mask w3
     float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
-    uint32_t mw[2][16];
+    uint32_t mw[16], mk[16];
+    load_sum32x4(mine, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {   // 32 units at a time: y, the mask, mask w3
-      float2 v[16];
-      load_sum32x4(lanes + 64 * half + 32 * h, v);
-      uint32_t mk[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int j = 64 * half + 32 * h + 2 * k;
-        const float2 w = *reinterpret_cast<const float2 *>(V.w3 + j), z2 = relu_bias(v[k], V.b2 + j);
-        acc[k & 1] = __ffma2_rn(w, z2, acc[k & 1]);
-        const uint32_t on = (z2.x > 0.0f ? 0x0000ffffu : 0u) | (z2.y > 0.0f ? 0xffff0000u : 0u);
-        mk[k] = on & 0x3f803f80u;   // 1.0 in bfloat16
-        mw[h][k] = on & __byte_perm(__float_as_uint(w.x), __float_as_uint(w.y), 0x7632);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        *reinterpret_cast<uint4 *>(chunk(mask + half * kBlock, row, 4 * h + c)) =
-            make_uint4(mk[4 * c], mk[4 * c + 1], mk[4 * c + 2], mk[4 * c + 3]);
+    for (int k = 0; k < 16; ++k) {
+      const int j = 32 * quarter + 2 * k;
+      const float2 w = *reinterpret_cast<const float2 *>(V.w3 + j), z2 = relu_bias(v[k], V.b2 + j);
+      acc[k & 1] = __ffma2_rn(w, z2, acc[k & 1]);
+      const uint32_t on = (z2.x > 0.0f ? 0x0000ffffu : 0u) | (z2.y > 0.0f ? 0xffff0000u : 0u);
+      mk[k] = on & 0x3f803f80u;   // 1.0 in bfloat16
+      mw[k] = on & __byte_perm(__float_as_uint(w.x), __float_as_uint(w.y), 0x7632);
     }
-    // y of the row: the two halves' sums
-    const float mine = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
-    if (half == 1) part[row] = mine;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      *reinterpret_cast<uint4 *>(chunk(mask + (quarter >> 1) * kBlock, row, 4 * (quarter & 1u) + c)) =
+          make_uint4(mk[4 * c], mk[4 * c + 1], mk[4 * c + 2], mk[4 * c + 3]);
+    // y of the row: the quarters' sums
+    part[quarter * kTileS + row] = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
     tc_before_sync();
     __syncthreads();   // (a2 has been read by all: its columns are free)
     tc_after_sync();
-    tmem_st16(lanes + kTm + 32 * half, mw[0]);
-    tmem_st16(lanes + kTm + 32 * half + 16, mw[1]);
-    if (half == 0) {
-      const float e = s0 + row < B ? mine + part[row] + V.b3 - target : 0.0f;
-      part[row] = e * inv_b;
+    tmem_st16(lanes + kTm + 16 * quarter, mw);
+    // (every quarter computes dy for itself; rows past the batch: 0, they add nothing)
+    const float y = ((part[row] + part[kTileS + row]) + (part[2 * kTileS + row] + part[3 * kTileS + row])) + V.b3;
+    const float e = s0 + row < B ? y - target : 0.0f, dy = e * inv_b;
+    if (quarter == 0) {
       lsum = fmaf(e, e, lsum);
-      gb3 += e * inv_b;
+      gb3 += dy;
     }
     tc_wait_st();
     tc_before_sync();
@@ -516,15 +517,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
         mma_ts(tm + 128 * (k >> 2), tm + kTm + 8 * k, dw2 + k * kRows16, idesc(kH, false, true), (k & 3u) > 0);
       tc_commit(&bar[0]);
     }
-    const float dy = part[row];   // (0 past the batch: such a row adds nothing)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {   // (layer 2's products have read z1)
-      float2 v[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = make_float2(dy * z1[16 * h + k].x, dy * z1[16 * h + k].y);
-      store_split32<false>(R, 2 * half + h, row, v);
-    }
-    if (half == 0) {
+    for (int k = 0; k < 16; ++k) v[k] = make_float2(dy * z1[k].x, dy * z1[k].y);
+    store_split32<false>(R, quarter, row, v);   // (layer 2's products have read z1)
+    if (quarter == 0) {
       uint32_t hi, mid, lo;
       split3<false>(make_float2(dy, 0.0f), hi, mid, lo);
       *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(hi << 16, mid | lo << 16, 0, 0);
@@ -533,16 +529,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
     ph0 ^= 1u;
     tc_after_sync();
+    load_sum32(mine, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float2 d[16];
-      load_sum32(lanes + 64 * half + 32 * h, d);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {   // d1
-        float2 &z = z1[16 * h + k];
-        z = make_float2(z.x > 0.0f ? dy * d[k].x : 0.0f, z.y > 0.0f ? dy * d[k].y : 0.0f);
-      }
-    }
+    for (int k = 0; k < 16; ++k)   // d1
+      z1[k] = make_float2(z1[k].x > 0.0f ? dy * v[k].x : 0.0f, z1[k].y > 0.0f ? dy * v[k].y : 0.0f);
     tc_before_sync();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -558,9 +548,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     ok = mbar_wait(&bar[1], ph1, &g_mlp_hdr) && ok;   // R and E are free
     ph1 ^= 1u;
     tc_after_sync();
-#pragma unroll
-    for (int h = 0; h < 2; ++h) store_split32<false>(R, 2 * half + h, row, z1 + 16 * h);
-    if (half == 0) *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(0x3f80u, 0, 0, 0);
+    store_split32<false>(R, quarter, row, z1);
+    if (quarter == 0) *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(0x3f80u, 0, 0, 0);
     fence_proxy_async_smem();
     tc_before_sync();
     __syncthreads();
@@ -577,50 +566,48 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     // meanwhile gW2 goes out: row j is this thread's lane
     const float w3 = V.w3[row];
     float2 dot = make_float2(0.0f, 0.0f);
+    load_sum32(mine, v);
+    {
+      uint32_t a[32];
+      tmem_ld32(mine + 256, a);
+      tc_wait_ld();
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float2 v[16];
-      load_sum32(lanes + 64 * half + 32 * h, v);
-      {
-        uint32_t a[32];
-        tmem_ld32(lanes + 256 + 64 * half + 32 * h, a);
-        tc_wait_ld();
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = __fadd2_rn(v[k], as_float2(a[2 * k], a[2 * k + 1]));
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const uint4 w = *reinterpret_cast<const uint4 *>(chunk(sm + GradSmem::w2 + half * kBlock, row, 4 * h + c));
-        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-        const float2 *g = v + 4 * c;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          dot = __ffma2_rn(as_float2(ww[k] << 16, ww[k] & 0xffff0000u), g[k], dot);
-        float *p = grad + kW2 + row * kH + 64 * half + 32 * h + 8 * c;
-        add4(p, w3 * g[0].x, w3 * g[0].y, w3 * g[1].x, w3 * g[1].y, gvec);
-        add4(p + 4, w3 * g[2].x, w3 * g[2].y, w3 * g[3].x, w3 * g[3].y, gvec);
-      }
+      for (int k = 0; k < 16; ++k) v[k] = __fadd2_rn(v[k], as_float2(a[2 * k], a[2 * k + 1]));
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint4 w =
+          *reinterpret_cast<const uint4 *>(chunk(sm + GradSmem::w2 + (quarter >> 1) * kBlock, row, 4 * (quarter & 1u) + c));
+      const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+      const float2 *g = v + 4 * c;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) dot = __ffma2_rn(as_float2(ww[k] << 16, ww[k] & 0xffff0000u), g[k], dot);
+      float *p = grad + kW2 + row * kH + 32 * quarter + 8 * c;
+      add4(p, w3 * g[0].x, w3 * g[0].y, w3 * g[1].x, w3 * g[1].y, gvec);
+      add4(p + 4, w3 * g[2].x, w3 * g[2].y, w3 * g[3].x, w3 * g[3].y, gvec);
+    }
+    part[quarter * kTileS + row] = dot.x + dot.y;   // (dy's sums have been read)
     ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
     ph0 ^= 1u;
     tc_after_sync();
+    __syncthreads();
     {
-      uint32_t a[32];
-      tmem_ld32(lanes + kTgW1 + 32 * half, a);
+      uint32_t a[16];
+      tmem_ld16(lanes + kTgW1 + 16 * quarter, a);
       tc_wait_ld();
 #pragma unroll
-      for (int k = 0; k < 32; k += 4)
-        add4(grad + kW1 + row * kIn + 32 * half + k, __uint_as_float(a[k]), __uint_as_float(a[k + 1]),
+      for (int k = 0; k < 16; k += 4)
+        add4(grad + kW1 + row * kIn + 16 * quarter + k, __uint_as_float(a[k]), __uint_as_float(a[k + 1]),
              __uint_as_float(a[k + 2]), __uint_as_float(a[k + 3]), gvec);
-      float gd = 0.0f;   // mask^T dy
-      if (half == 0) {
-        tmem_ld32(lanes + kTgB, a);
+      if (quarter == 0) {
+        tmem_ld16(lanes + kTgB, a);
         tc_wait_ld();
-        gd = (__uint_as_float(a[1]) + __uint_as_float(a[2])) + __uint_as_float(a[3]);
+        const float gd = (__uint_as_float(a[1]) + __uint_as_float(a[2])) + __uint_as_float(a[3]);   // mask^T dy
+        const float d = (part[row] + part[kTileS + row]) + (part[2 * kTileS + row] + part[3 * kTileS + row]);
         atomicAdd(&grad[kB1 + row], __uint_as_float(a[0]));
         atomicAdd(&grad[kB2 + row], w3 * gd);
+        atomicAdd(&grad[kW3 + row], fmaf(V.b2[row], gd, d));
       }
-      atomicAdd(&grad[kW3 + row], fmaf(V.b2[row], gd, dot.x + dot.y));   // each half its units
     }
     store_x<kGradThreads>(sm + GradSmem::x, xr);
     fence_proxy_async_smem();
@@ -629,7 +616,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     if (!ok) break;   // a wait gave up (recorded): the whole block leaves
     tc_after_sync();
   }
-  if (half == 0) {
+  if (quarter == 0) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       lsum += __shfl_xor_sync(FULL, lsum, o);
