@@ -356,7 +356,7 @@ def run_esc(args):
             "roofline": {"bound": "hbm", "achieved": scan_achieved, "peak": peak, "unit": "GB/s",
                          "frac": scan_achieved / peak, "traffic": profiled_traffic("count", args.rows),
                          "kernel": "esc::scan_kernel", "peak_source": peak_src,
-                         "measured_on": "the same 200 predicates counted (one launch per call: scan_kernel, or "
+                         "measured_on": "the same 200 predicates counted (clear_kernel and scan_kernel, or "
                                         "const_kernel for a program folded to a constant), CUDA events around each call",
                          "algorithmic_bytes_per_launch": sum(scan_bytes) / len(scan_bytes)},
             "roofline_call": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -367,8 +367,9 @@ def run_esc(args):
                     "d2h_bytes_per_step": host_counts.numel() * 8,
                     "what": "per step: the table copied from pinned host memory, 200 sub-queries through the "
                             "C ABI, counts read back; the next step's copy overlaps this step's sub-queries"},
-            # scan_kernel + write_kernel per sub-query; const_kernel alone for a program folded to a constant
-            "gpu_launches": K * sum(1 if not r else 2 for r in refs),
+            # clear_kernel + scan_kernel + write_kernel per sub-query; clear_kernel + const_kernel for a program
+            # folded to a constant
+            "gpu_launches": K * sum(2 if not r else 3 for r in refs),
             "clocks": clk.summary(),
             "cpu_baseline": cpu,
         }
