@@ -13,16 +13,19 @@
 //    split its domain into intervals on which every test is constant;
 //    build_kernel evaluates, for each operand and interval, the tests of all
 //    boxes at one value of the interval: a row of bits, one per box.
-//  * box_kernel finds each row's interval in every operand (binary search, or
-//    the value itself for u8), ANDs the operands' bit rows, 32 boxes per word,
-//    and counts the words vertically: bit-sliced counters fed by a carry-save
-//    tree, two logic instructions per adder.
+//  * box_kernel finds each row's interval in every operand (a bucket of equal
+//    width, then binary search among its cuts; the value itself for u8), ANDs
+//    the operands' bit rows, 32 boxes per word, and counts the words vertically:
+//    bit-sliced counters fed by a carry-save tree, two logic instructions per
+//    adder.
 // What bounds it: for many boxes, the table rows' traffic through L1 (a row of
 // 2048 predicates is about 420 bytes per operand: 65 % of L1's throughput,
-// 59 % of it hits); for few, the instructions of the binary searches (63 % of
-// the issue slots).  Measured on the 8M-row skewed table, interpreted before
-// and looked up now: 16 predicates 304 -> 143 us, 32 555 -> 199, 64 1446 ->
-// 270, 256 5.45 ms -> 0.66, 2048 42.0 ms -> 2.88.
+// 59 % of it hits); for few, the instructions of the searches (63 % of the
+// issue slots without buckets).  Measured on the 8M-row skewed table,
+// interpreted before and looked up now: 16 predicates 304 -> 121 us, 32 555 ->
+// 169, 64 1446 -> 220.  Buckets took the searches from 138, 195 and 265 us in
+// these cases, and on 20M rows from 1.58 to 1.29 ms for 256 predicates, 2.97 to
+// 2.24 for 512, 7.29 to 6.35 for 2048.
 // Predicates that do not decompose within the limits below are interpreted
 // (shared_kernel in esc_scan.cu).
 #include <cuda_runtime.h>
@@ -47,6 +50,13 @@ constexpr int kPlanes = 11;             // bit planes of a vertical counter
 constexpr uint32_t kMaxPending = (1u << kPlanes) - 1 - 8;
 constexpr uint32_t kCutSmem = 16 * 1024;    // cuts copied to shared memory up to this size
 constexpr uint32_t kTableSmem = 40 * 1024;  // the same for the bit table
+// Bucket tables (see `bucket_search`): at most this many bytes for all operands
+// and buckets for one, and about this many buckets per cut.  (512 to 2048 and 4
+// to 32: within 2 % of one another, except that the larger tables cost a
+// resident block at 32 predicates, 169 -> 185 us.)
+constexpr uint32_t kBucketBytes = 16 * 1024;
+constexpr uint32_t kMaxBuckets = 1024;
+constexpr uint32_t kBucketsPerCut = 8;
 constexpr int kBoxStages = 2;           // tiles of columns in flight or in use
 
 // How an operand's interval is found: the value itself (u8), or by searching
@@ -62,6 +72,11 @@ struct Operand {
   uint32_t steps;         // binary-search steps; 2^steps - 1 padded cuts
   uint32_t cut_off;       // byte offset of the cuts
   uint32_t table_off;     // byte offset of interval 0's bit row
+  // buckets of equal width (2^shift) over the cuts' values (kind OPD_32; bsteps ~0: none)
+  uint32_t bsteps;        // binary-search steps left in a bucket
+  uint32_t bucket_off;    // byte offset of the buckets
+  int32_t base, top;      // one below the first cut; the last cut
+  uint32_t shift;
   // udf: modulus, its remainder constants (below 2^16: M, K; else mult, sh1, sh2)
   uint32_t K;
   int32_t sh1, sh2;
@@ -87,9 +102,11 @@ struct BoxLaunch {
   uint32_t lanes;             // lanes that share a row (power of two)
   uint32_t chunks;            // passes over a bit row: VEC * lanes words each
   uint32_t cuts_in_smem;
+  uint32_t bucket_bytes;
   // byte offsets in shared memory (first the stages)
-  uint32_t smem_offs, smem_cnt, smem_cut, smem_table, smem_bar;
+  uint32_t smem_offs, smem_cnt, smem_cut, smem_table, smem_bar, smem_bucket;
   const uint8_t *cuts;        // sorted, padded
+  const uint8_t *buckets;     // u16 each
   uint8_t *table;
   const uint32_t *pred_of_box;
   const uint32_t *lane_ops;   // per 4 words of the bit row: operands their boxes test (bits)
@@ -288,14 +305,47 @@ __device__ __forceinline__ void search(const uint8_t *cuts, uint32_t steps, uint
   for (int k = 0; k < R; ++k) pos[k] = min(pos[k], ncuts);   // padding equals the largest value
 }
 
+// The same with a table of buckets: the value's bucket gives the number of cuts
+// before it (with buckets of one value: up to it), and the search goes on among
+// the bucket's own cuts, `bsteps` halvings for the fullest one.  Later buckets'
+// cuts lie above the value, so halvings past the bucket's end find nothing.
+template <int R>
+__device__ __forceinline__ void bucket_search(const Operand &o, const uint8_t *cuts, const uint8_t *buckets,
+                                              const int32_t (&v)[R], uint32_t (&pos)[R]) {
+  const int32_t *cut = reinterpret_cast<const int32_t *>(cuts + o.cut_off) - 1;
+  const uint16_t *first = reinterpret_cast<const uint16_t *>(buckets + o.bucket_off);
+  int32_t w[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    w[k] = max(o.base, min(v[k], o.top));
+    pos[k] = first[((uint32_t)w[k] - (uint32_t)o.base) >> o.shift];
+  }
+  for (uint32_t h = 1u << o.bsteps >> 1; h; h >>= 1) {
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const uint32_t t = pos[k] + h;
+      if (cut[t] <= w[k]) pos[k] = t;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) pos[k] = min(pos[k], o.ncuts);
+}
+
+template <int R>
+__device__ __forceinline__ void search32(const Operand &o, const uint8_t *cuts, const uint8_t *buckets,
+                                         const int32_t (&v)[R], uint32_t (&pos)[R]) {
+  if (o.bsteps != ~0u) bucket_search<R>(o, cuts, buckets, v, pos);
+  else search<int32_t, R>(cuts + o.cut_off, o.steps, o.ncuts, v, pos);
+}
+
 __device__ __forceinline__ int32_t saturate32(int64_t v) {
   return (int32_t)max((int64_t)INT32_MIN, min((int64_t)INT32_MAX, v));
 }
 
 // The intervals of operand o of R rows of a staged tile: rows row + k * kBoxThreads.
 template <int R>
-__device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage, const uint8_t *cuts, uint32_t row,
-                                          uint32_t (&pos)[R]) {
+__device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage, const uint8_t *cuts, const uint8_t *buckets,
+                                          uint32_t row, uint32_t (&pos)[R]) {
   const uint8_t *a = stage + o.a;
   if (o.kind == OPD_U8) {
 #pragma unroll
@@ -311,7 +361,7 @@ __device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage
 #pragma unroll
       for (int k = 0; k < R; ++k) v[k] = reinterpret_cast<const uint16_t *>(a)[row + k * kBoxThreads];
     }
-    search<int32_t, R>(cuts + o.cut_off, o.steps, o.ncuts, v, pos);
+    search32<R>(o, cuts, buckets, v, pos);
     return;
   }
   long long v[R];
@@ -327,7 +377,7 @@ __device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage
     int32_t w[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) w[k] = saturate32(v[k]);
-    search<int32_t, R>(cuts + o.cut_off, o.steps, o.ncuts, w, pos);
+    search32<R>(o, cuts, buckets, w, pos);
   }
 }
 
@@ -484,6 +534,7 @@ __global__ void __launch_bounds__(kBoxThreads, VEC == 4 ? 2 : 3) box_rows_kernel
   for (uint32_t i = threadIdx.x; i < L.nboxes; i += kBoxThreads) cnt[i] = 0;
   copy16(sm + L.smem_cut, L.cuts, L.cut_bytes);
   copy16(sm + L.smem_table, L.table, L.table_bytes);
+  copy16(sm + L.smem_bucket, L.buckets, L.bucket_bytes);
   const uint8_t *cuts = sm + L.smem_cut, *table = sm + L.smem_table;
   uint32_t p[VEC][kPlanes];
 #pragma unroll
@@ -505,7 +556,7 @@ __global__ void __launch_bounds__(kBoxThreads, VEC == 4 ? 2 : 3) box_rows_kernel
     for (int c = 0; c < L.nop; ++c) {
       const Operand &o = L.op[c];
       uint32_t pos[kRows];
-      intervals<kRows>(o, stage, cuts, threadIdx.x, pos);
+      intervals<kRows>(o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
 #pragma unroll
       for (int k = 0; k < kRows; ++k) {
         uint32_t off = o.table_off + pos[k] * (4u * VEC);
@@ -550,6 +601,7 @@ __global__ void __launch_bounds__(kBoxThreads, 2) box_words_kernel(const __grid_
   TileRing ring;
   ring.start(L, sm, L.chunks);
   for (uint32_t i = threadIdx.x; i < L.nboxes; i += kBoxThreads) cnt[i] = 0;
+  copy16(sm + L.smem_bucket, L.buckets, L.bucket_bytes);
   const uint8_t *cuts = L.cuts;
   if (L.cuts_in_smem) {
     copy16(sm + L.smem_cut, L.cuts, L.cut_bytes);
@@ -583,7 +635,7 @@ __global__ void __launch_bounds__(kBoxThreads, 2) box_words_kernel(const __grid_
     for (int c = 0; c < L.nop; ++c) {
       const Operand &o = L.op[c];
       uint32_t pos[2];
-      intervals<2>(o, stage, cuts, threadIdx.x, pos);
+      intervals<2>(o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         uint32_t off = o.table_off + pos[k] * L.stride;
@@ -886,6 +938,34 @@ void sort_boxes(BoxPlan *P, std::vector<uint32_t> &lane_ops) {
   P->boxes.swap(sorted);
 }
 
+// An operand's buckets, where they save at least two halvings (a bucket costs
+// about as much as one): the smallest power-of-two width that gives at most
+// `most` of them.  `cuts` in any order; appended to `out`.
+void make_buckets(Operand &o, const std::vector<int64_t> &cuts, uint32_t most, std::vector<uint16_t> &out) {
+  o.bsteps = ~0u;
+  if (o.kind != OPD_32 || o.ncuts < 3 || o.ncuts > 65535 || most < 8) return;
+  const auto mm = std::minmax_element(cuts.begin(), cuts.end());
+  const int64_t base = *mm.first - 1, top = *mm.second;   // (cuts lie above the least 32-bit value)
+  const uint64_t span = (uint64_t)(top - base);
+  uint32_t shift = 0;
+  while ((span >> shift) + 1 > most) ++shift;
+  const uint32_t n = (uint32_t)(span >> shift) + 1;
+  std::vector<uint32_t> before(n + 1, 0);   // cuts in buckets before each
+  for (int64_t v : cuts) ++before[(size_t)((uint64_t)(v - base) >> shift) + 1];
+  const uint32_t fullest = *std::max_element(before.begin(), before.end());
+  uint32_t bsteps = 0;
+  if (shift)
+    while ((1ull << bsteps) - 1 < fullest) ++bsteps;
+  if (bsteps + 2 > o.steps) return;
+  for (uint32_t k = 0; k < n; ++k) before[k + 1] += before[k];
+  o.bsteps = bsteps;
+  o.base = (int32_t)base;
+  o.top = (int32_t)top;
+  o.shift = shift;
+  o.bucket_off = (uint32_t)(out.size() * 2);
+  for (uint32_t k = 0; k < n; ++k) out.push_back((uint16_t)before[shift ? k : k + 1]);
+}
+
 }  // namespace
 
 esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long *counts, ScratchHdr *hdr,
@@ -935,6 +1015,12 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   size_t many = 0;
   for (auto &h : P->ops) many += h.cuts.size();
   const bool gpu_sort = many > 2048;
+  uint32_t searched = 0;   // operands that may have buckets
+  for (auto &h : P->ops) searched += h.col2 >= 0 || t->dtypes[h.col] != ESC_U8;
+  uint32_t most_buckets = kMaxBuckets;
+  while (most_buckets * searched * 2 > kBucketBytes) most_buckets /= 2;
+  std::vector<uint16_t> buckets;
+  std::vector<uint32_t> padded_cuts((size_t)L.nop);
   for (int c = 0; c < L.nop; ++c) {
     HostOperand &h = P->ops[order[c]];
     Operand &o = L.op[c];
@@ -989,7 +1075,13 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
     }
     o.ncuts = (uint32_t)h.cuts.size();
     while ((1ull << o.steps) - 1 < o.ncuts) ++o.steps;
-    const uint32_t padded = (1u << o.steps) - 1, w = o.kind == OPD_64 ? 8u : 4u;
+    uint32_t per_cut = 8;
+    while (per_cut < o.ncuts * kBucketsPerCut) per_cut *= 2;
+    make_buckets(o, h.cuts, std::min(most_buckets, per_cut), buckets);
+    // every halving reads inside the padding, also those that start at a bucket's first cut
+    const uint32_t padded = std::max((1u << o.steps) - 1, o.bsteps == ~0u ? 0u : o.ncuts + (1u << o.bsteps) - 1);
+    const uint32_t w = o.kind == OPD_64 ? 8u : 4u;
+    padded_cuts[c] = padded;
     o.cut_off = (uint32_t)cut_bytes;
     if (job) {
       job->padded = padded;
@@ -1002,6 +1094,7 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   }
   if (intervals * (words + 3) * 4 > kMaxTableBytes) return ESC_OK;   // too large to pay: the caller interprets
   L.cut_bytes = round16(cut_bytes);
+  L.bucket_bytes = round16(buckets.size() * 2);
   // shared memory, and with it the kernel: rows in registers when the boxes
   // fit a thread's words and cuts and table fit beside the stages
   const uint32_t row_bytes = L.stage_bytes;
@@ -1023,10 +1116,11 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   int vec = words <= 1 ? 1 : words <= 2 ? 2 : 4;
   uint64_t table_bytes = intervals * vec * 4;
   const bool by_row = words <= 4 && L.cut_bytes <= kCutSmem && table_bytes <= kTableSmem &&
-                      smem + L.cut_bytes + table_bytes + 32 <= (uint64_t)kMaxBoxSmem;
+                      smem + L.cut_bytes + table_bytes + L.bucket_bytes + 48 <= (uint64_t)kMaxBoxSmem;
   if (by_row) {
     L.smem_cut = take(L.cut_bytes);
     L.smem_table = take(table_bytes);
+    L.smem_bucket = take(L.bucket_bytes);
   } else {
     vec = 4;
     L.lanes = 1;
@@ -1035,6 +1129,7 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
     table_bytes = intervals * ((words + 3) & ~3u) * 4;
     layout(kTile);
     L.smem_offs = take((uint64_t)kTile * L.nopp * 4);
+    L.smem_bucket = take(L.bucket_bytes);
     if (L.cut_bytes <= kCutSmem && smem + L.cut_bytes <= (uint32_t)kMaxBoxSmem) {
       L.cuts_in_smem = 1;
       L.smem_cut = take(L.cut_bytes);
@@ -1060,7 +1155,7 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
                  a_box = place((uint64_t)nboxes * 8), a_pred = place((uint64_t)nboxes * 4),
                  a_lane = place(lane_ops.size() * 4),
                  a_pool = place(P->pool.size() * 8 + 8), a_jobs = place(jobs.size() * sizeof(SortJob) + 4),
-                 a_uns = place(unsorted.size() * 8 + 8), a_cuts = place(L.cut_bytes + 16), upload = at,
+                 a_uns = place(unsorted.size() * 8 + 8), a_buckets = place(L.bucket_bytes + 16), a_cuts = place(L.cut_bytes + 16), upload = at,
                  a_table = place(round16(table_bytes));
   void *mem = nullptr;
   esc_status s = alloc_async(&mem, at, st);
@@ -1081,11 +1176,12 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   put(a_pool, P->pool.data(), P->pool.size() * 8);
   put(a_jobs, jobs.data(), jobs.size() * sizeof(SortJob));
   put(a_uns, unsorted.data(), unsorted.size() * 8);
+  put(a_buckets, buckets.data(), buckets.size() * 2);
   for (int c = 0; c < L.nop; ++c) {   // cuts sorted here, padded (those sorted on the GPU are overwritten there)
     const Operand &o = L.op[c];
     if (o.kind == OPD_U8) continue;
     const std::vector<int64_t> &cuts = P->ops[order[c]].cuts;
-    const uint32_t padded = (1u << o.steps) - 1;
+    const uint32_t padded = padded_cuts[c];
     for (uint32_t k = 0; k < padded; ++k) {
       if (o.kind == OPD_64) {
         const int64_t v = k < o.ncuts ? cuts[k] : INT64_MAX;
@@ -1098,6 +1194,7 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   }
   L.cuts = dev + a_cuts;
   L.table = dev + a_table;
+  L.buckets = dev + a_buckets;
   L.lane_ops = reinterpret_cast<const uint32_t *>(dev + a_lane);
   L.pred_of_box = reinterpret_cast<const uint32_t *>(dev + a_pred);
   L.counts = counts;
