@@ -19,13 +19,13 @@
 //    bit-sliced counters fed by a carry-save tree, two logic instructions per
 //    adder.
 // What bounds it: for many boxes, the table rows' traffic through L1 (a row of
-// 2048 predicates is about 420 bytes per operand: 65 % of L1's throughput,
-// 59 % of it hits); for few, the instructions of the searches (63 % of the
-// issue slots without buckets).  Measured on the 8M-row skewed table,
-// interpreted before and looked up now: 16 predicates 304 -> 121 us, 32 555 ->
-// 169, 64 1446 -> 220.  Buckets took the searches from 138, 195 and 265 us in
-// these cases, and on 20M rows from 1.58 to 1.29 ms for 256 predicates, 2.97 to
-// 2.24 for 512, 7.29 to 6.35 for 2048.
+// 2048 predicates is about 420 bytes per operand: 50 % of L1's throughput, 46 %
+// of it hits, and the latency shows at 16 warps per SM); for few, the
+// instructions that find the intervals (67 % of the issue slots).  Measured on
+// the 8M-row skewed table, interpreted before and looked up now: 16 predicates
+// 304 -> 121 us, 32 555 -> 168, 64 1446 -> 220, 256 5.45 ms -> 0.52, 2048 42.0
+// ms -> 2.26.  Without buckets the first three take 138, 195 and 265 us, and on
+// 20M rows 256 predicates 1.58 ms (1.29 with), 512 2.97 (2.24), 2048 7.29 (6.35).
 // Predicates that do not decompose within the limits below are interpreted
 // (shared_kernel in esc_scan.cu).
 #include <cuda_runtime.h>

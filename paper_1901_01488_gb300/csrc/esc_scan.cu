@@ -2513,10 +2513,15 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
 // two launches more (about 25 us) and the rows' intervals, whatever n;
 // interpreting costs about 2.3 us per predicate and million rows, and from 17
 // predicates on about 1 us per predicate to copy their programs.  Both
-// measured, lookup / interpreter, us: 8M rows: 4 predicates 111 / 80, 8 154 /
-// 148, 12 162 / 239, 16 138 / 302, 32 195 / 554; 1M: 8 61 / 38, 12 58 / 53, 16
-// 54 / 64, 32 73 / 115; 100K: 16 46 / 37, 32 53 / 66; 10K: 32 52 / 54, 64 59 / 92.
-inline bool lookup_pays(int32_t n, uint64_t rows) { return n >= 12 && (n >= 32 || rows * (uint64_t)n >= 16000000u); }
+// measured with three sets of predicates, lookup / interpreter, us: 60M rows: 6
+// predicates 614-825 / 593-976, 8 802-815 / 819-1173, 10 610-816 / 1229-1506;
+// 8M: 8 145-148 / 129-177, 10 119-148 / 185-222, 12 143-147 / 235-256, 16
+// 122-152 / 285-301; 1M: 10 51-56 / 44-51, 12 56 / 52-55, 16 52-60 / 62-64, 32
+// 67-70 / 102-110; 100K: 16 41-47 / 36-38, 32 51 / 55-61.
+inline bool lookup_pays(int32_t n, uint64_t rows) {
+  const uint64_t work = rows * (uint64_t)n;
+  return n >= 32 || (n >= 12 && work >= 16000000u) || (n >= 8 && work >= 80000000u);
+}
 
 // One shared scan: `n` count-only predicates of table t whose read columns
 // (union `ucols`, table column indices) fit one stage layout.  Predicates that

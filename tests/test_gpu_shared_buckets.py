@@ -59,3 +59,18 @@ def test_against_counting(kind, npred):
     dev = torch.full((npred,), -1, dtype=torch.int64, device="cuda")
     esc.esc_selectivity_shared_async(t.handle, ps.handles, dev)
     assert dev.tolist() == want
+
+
+@pytest.mark.parametrize("rows", [9_999_999, 10_000_000])
+def test_eight_predicates(rows):
+    """On both sides of the size from which eight predicates are looked up."""
+    from paper_1901_01488_gb300 import esc
+    rng = np.random.default_rng(8)
+    cols = {"a": rng.integers(-1000, 1000, rows).astype(np.int32), "b": rng.integers(0, 256, rows).astype(np.uint8)}
+    t = esc.Table(as_columns(cols, "cuda"), rows)
+    texts = [f"a BETWEEN {-900 + 100 * k} AND {37 * k} AND b >= {9 * k}" for k in range(8)]
+    ps = esc.PredicateSet(t, texts)
+    dev = torch.full((8,), -1, dtype=torch.int64, device="cuda")
+    esc.esc_selectivity_shared_async(t.handle, ps.handles, dev)
+    assert dev.tolist() == [int(((cols["a"] >= -900 + 100 * k) & (cols["a"] <= 37 * k) & (cols["b"] >= 9 * k)).sum())
+                            for k in range(8)]
