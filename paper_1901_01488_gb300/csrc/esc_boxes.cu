@@ -1129,6 +1129,10 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
     table_bytes = intervals * ((words + 3) & ~3u) * 4;
     layout(kTile);
     L.smem_offs = take((uint64_t)kTile * L.nopp * 4);
+    if (smem + L.bucket_bytes > (uint32_t)kMaxBoxSmem) {   // (16 i64 columns, 24 operands, 8192 boxes leave 12,272 bytes)
+      L.bucket_bytes = 0;
+      for (int c = 0; c < L.nop; ++c) L.op[c].bsteps = ~0u;
+    }
     L.smem_bucket = take(L.bucket_bytes);
     if (L.cut_bytes <= kCutSmem && smem + L.cut_bytes <= (uint32_t)kMaxBoxSmem) {
       L.cuts_in_smem = 1;
@@ -1155,7 +1159,8 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
                  a_box = place((uint64_t)nboxes * 8), a_pred = place((uint64_t)nboxes * 4),
                  a_lane = place(lane_ops.size() * 4),
                  a_pool = place(P->pool.size() * 8 + 8), a_jobs = place(jobs.size() * sizeof(SortJob) + 4),
-                 a_uns = place(unsorted.size() * 8 + 8), a_buckets = place(L.bucket_bytes + 16), a_cuts = place(L.cut_bytes + 16), upload = at,
+                 a_uns = place(unsorted.size() * 8 + 8), a_buckets = place(buckets.size() * 2 + 16),
+                 a_cuts = place(L.cut_bytes + 16), upload = at,
                  a_table = place(round16(table_bytes));
   void *mem = nullptr;
   esc_status s = alloc_async(&mem, at, st);

@@ -74,3 +74,32 @@ def test_eight_predicates(rows):
     esc.esc_selectivity_shared_async(t.handle, ps.handles, dev)
     assert dev.tolist() == [int(((cols["a"] >= -900 + 100 * k) & (cols["a"] <= 37 * k) & (cols["b"] >= 9 * k)).sum())
                             for k in range(8)]
+
+
+def test_largest_pass():
+    """A pass at all its limits: 16 i64 columns, 24 operands, 8192 boxes, 256
+    buckets for every operand, more shared memory than there is."""
+    from paper_1901_01488_gb300 import esc
+    rows, top = 3001, 1 << 20
+    rng = np.random.default_rng(24)
+    names = [f"c{k}" for k in range(16)]
+    cols = {n: rng.integers(-5, top + 5, rows) for n in names}
+    t = esc.Table(as_columns(cols, "cuda"), rows)
+    m = 1 << 21
+    values = [(n, cols[n]) for n in names]
+    values += [(f"udf({names[2 * k]}, {names[2 * k + 1]}, {m})", np.fmod(cols[names[2 * k]] * cols[names[2 * k + 1]], m))
+               for k in range(8)]
+    texts, want = [], []
+    for k in range(2048):
+        ops = [values[(4 * k + j) % 24] for j in range(4)]
+        lo = [1 if k < 6 else int(rng.integers(1, top - 2)) for _ in ops]    # the first six meet every operand
+        hi = [top - 2 if k < 6 else int(rng.integers(x, top - 1)) for x in lo]
+        texts.append(" OR ".join(f"{n} BETWEEN {a} AND {b}" for (n, _), a, b in zip(ops, lo, hi)))
+        hit = np.zeros(rows, bool)
+        for (_, v), a, b in zip(ops, lo, hi):
+            hit |= (v >= a) & (v <= b)
+        want.append(int(hit.sum()))
+    ps = esc.PredicateSet(t, texts)
+    dev = torch.full((2048,), -1, dtype=torch.int64, device="cuda")
+    esc.esc_selectivity_shared_async(t.handle, ps.handles, dev)
+    assert dev.tolist() == want
