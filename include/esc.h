@@ -320,7 +320,9 @@ esc_status esc_mlp_forward(const uint16_t *x_bf16, uint64_t batch, const uint16_
 
 /* Adds to grad[ESC_MLP_PARAMS] the gradient of mean_i (y_i - target_i)^2
  * over the batch, and to *loss_sum the sum of squared errors.  The caller
- * zeroes both beforehand. */
+ * zeroes both beforehand.  A sample with an infinite or NaN residual makes
+ * non-finite only the entries it contributes to: a unit it leaves inactive
+ * gets nothing from it. */
 esc_status esc_mlp_grad(const uint16_t *x_bf16, const float *target, uint64_t batch,
                         const uint16_t *w_bf16, const float *params, float *grad, float *loss_sum,
                         void *stream);

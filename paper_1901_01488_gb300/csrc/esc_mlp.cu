@@ -18,7 +18,10 @@
 // gradient is the outer product of dy and w3 under the ReLU mask:
 //   d1 = dy (mask w3) W2,   gW2 = w3 (mask^T (dy z1)),   gb2 = w3 (mask^T dy),
 //   gw3[j] = sum_k W2[j][k] (mask^T (dy z1))[j][k] + b2[j] (mask^T dy)[j],
-// so that only z1, dy z1 and d1 need the split.
+// so that only z1, dy z1 and d1 need the split.  A factor of these sums over
+// samples that is infinite or NaN would reach every unit, active or not (0
+// times it is NaN), so such samples take part in them with zeros and are added
+// by plain arithmetic (add_sample): only what they reach becomes non-finite.
 //
 // Shared-memory operands are rows of 128 bytes with 128-byte swizzle (the
 // 16-byte chunk c of row r at c ^ (r % 8)), 64 columns a block of 16 KB per 128
@@ -29,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -402,7 +406,8 @@ constexpr uint32_t kTgB = 384, kTm = 448, kTgW1 = 448;
 struct GradSmem {
   static constexpr uint32_t w1 = 0, w2 = kBlock, x = 3 * kBlock, e = 4 * kBlock, mask = 5 * kBlock, r = 7 * kBlock,
                             vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * 4 * kTileS, tmem = bar + 16,
-                            total = tmem + 16;
+                            bad = tmem + 16, bad_dy = bad + 16,
+                            total = bad_dy + 4 * kTileS;
 };
 
 __device__ __forceinline__ void add4(float *p, float a, float b, float c, float d, bool vec) {
@@ -416,6 +421,47 @@ __device__ __forceinline__ void add4(float *p, float a, float b, float c, float 
   }
 }
 
+// Value i of a row of an operand block (two blocks for 128 columns).
+__device__ __forceinline__ float operand(const uint8_t *blocks, uint32_t row, uint32_t i) {
+  const uint8_t *b = blocks + (i >> 6) * kBlock + row * 128u + ((((i >> 3) & 7u) ^ (row & 7u)) << 4) + 2u * (i & 7u);
+  return bf(*reinterpret_cast<const uint16_t *>(b));
+}
+
+// Adds one sample's gradient (the tile's row r) by plain arithmetic, unit by
+// unit: for samples with an infinity or NaN among the products' factors.  Those
+// are left out of the products, where 0 times such a factor would reach every
+// unit, active or not.  `s`: 384 floats of scratch in shared memory; the whole
+// block calls.
+__device__ __noinline__ void add_sample(const uint8_t *sm, const MlpVectors &V, float *s, uint32_t r, float dy, float *grad) {
+  const uint8_t *w1 = sm + GradSmem::w1, *w2 = sm + GradSmem::w2, *x = sm + GradSmem::x;
+  float *z1 = s, *d2 = s + kH, *d1 = s + 2 * kH;
+  const uint32_t j = threadIdx.x & 127u, quarter = threadIdx.x >> 7;
+  if (quarter == 0) {
+    float a = V.b1[j];
+    for (uint32_t m = 0; m < kIn; ++m) a = fmaf(operand(w1, j, m), operand(x, r, m), a);
+    z1[j] = fmaxf(a, 0.0f);
+  }
+  __syncthreads();
+  if (quarter == 0) {
+    float a = V.b2[j];
+    for (uint32_t k = 0; k < kH; ++k) a = fmaf(operand(w2, j, k), z1[k], a);
+    d2[j] = a > 0.0f ? dy * V.w3[j] : 0.0f;
+    atomicAdd(&grad[kB2 + j], d2[j]);
+    atomicAdd(&grad[kW3 + j], dy * fmaxf(a, 0.0f));
+  }
+  __syncthreads();
+  for (uint32_t k = 32 * quarter; k < 32 * quarter + 32; ++k) atomicAdd(&grad[kW2 + j * kH + k], d2[j] * z1[k]);
+  if (quarter == 0) {
+    float g = 0.0f;
+    for (uint32_t i = 0; i < kH; ++i) g = fmaf(operand(w2, i, j), d2[i], g);
+    d1[j] = z1[j] > 0.0f ? g : 0.0f;
+    atomicAdd(&grad[kB1 + j], d1[j]);
+  }
+  __syncthreads();
+  for (uint32_t m = 16 * quarter; m < 16 * quarter + 16; ++m) atomicAdd(&grad[kW1 + j * kIn + m], d1[j] * operand(x, r, m));
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_t *x, const float *t, uint64_t B,
                                                                    const uint16_t *wbf, const float *pf, float *grad,
                                                                    float *loss_sum) {
@@ -425,6 +471,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [2]
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + GradSmem::tmem);
   uint8_t *R = sm + GradSmem::r, *E = sm + GradSmem::e, *mask = sm + GradSmem::mask;
+  uint32_t *bad = reinterpret_cast<uint32_t *>(sm + GradSmem::bad);   // the tile's samples left to add_sample (bits)
+  float *bad_dy = reinterpret_cast<float *>(sm + GradSmem::bad_dy);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, quarter = warp >> 2, row = threadIdx.x & 127u;
   const bool vec = ((uintptr_t)x & 15u) == 0, gvec = ((uintptr_t)grad & 15u) == 0;
   uint4 xr[2];
@@ -433,6 +481,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+    bad[0] = bad[1] = bad[2] = bad[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   load_weights<kGradThreads>(sm + GradSmem::w1, sm + GradSmem::w2, V, wbf, pf);
@@ -520,6 +569,9 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = make_float2(dy * z1[k].x, dy * z1[k].y);
     store_split32<false>(R, quarter, row, v);   // (layer 2's products have read z1)
+    float2 odd = make_float2(dy * 0.0f, 0.0f);   // NaN once a factor is infinite or NaN
+#pragma unroll
+    for (int k = 0; k < 16; ++k) odd = __ffma2_rn(v[k], make_float2(0.0f, 0.0f), odd);
     if (quarter == 0) {
       uint32_t hi, mid, lo;
       split3<false>(make_float2(dy, 0.0f), hi, mid, lo);
@@ -533,8 +585,24 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
 #pragma unroll
     for (int k = 0; k < 16; ++k)   // d1
       z1[k] = make_float2(z1[k].x > 0.0f ? dy * v[k].x : 0.0f, z1[k].y > 0.0f ? dy * v[k].y : 0.0f);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) odd = __ffma2_rn(z1[k], make_float2(0.0f, 0.0f), odd);
+    const bool left_out = !(odd.x + odd.y == 0.0f);
     tc_before_sync();
-    __syncthreads();
+    if (__syncthreads_or(left_out)) {   // those samples' operands become 0; add_sample makes up for them below
+      if (left_out) atomicOr(&bad[row >> 5], 1u << (row & 31u));
+      if (quarter == 0) bad_dy[row] = dy;
+      __syncthreads();
+      if ((bad[row >> 5] >> (row & 31u)) & 1u) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) z1[k] = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+        for (uint32_t c = quarter; c < 6 * 8 + 1; c += 4)   // its 16-byte chunks in R, and the one in use in E
+          *reinterpret_cast<uint4 *>(c < 48 ? chunk(R + (c >> 3) * kBlock, row, c & 7u) : chunk(E, row, 0)) = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
+      }
+      __syncthreads();
+    }
     if (threadIdx.x == 0) {
       tc_after_sync();
       for (int p = 2; p >= 0; --p)         // mask^T (dy z1): every third 16 samples per accumulator
@@ -586,6 +654,12 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       add4(p, w3 * g[0].x, w3 * g[0].y, w3 * g[1].x, w3 * g[1].y, gvec);
       add4(p + 4, w3 * g[2].x, w3 * g[2].y, w3 * g[3].x, w3 * g[3].y, gvec);
     }
+    if (!(fabsf(dot.x + dot.y) <= FLT_MAX)) {   // a weight is infinite or NaN: 0 where no sample activates the unit
+      float any = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) any += fabsf(v[k].x) + fabsf(v[k].y);
+      if (any == 0.0f) dot = make_float2(0.0f, 0.0f);
+    }
     part[quarter * kTileS + row] = dot.x + dot.y;   // (dy's sums have been read)
     ok = mbar_wait(&bar[0], ph0, &g_mlp_hdr) && ok;
     ph0 ^= 1u;
@@ -606,8 +680,15 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
         const float d = (part[row] + part[kTileS + row]) + (part[2 * kTileS + row] + part[3 * kTileS + row]);
         atomicAdd(&grad[kB1 + row], __uint_as_float(a[0]));
         atomicAdd(&grad[kB2 + row], w3 * gd);
-        atomicAdd(&grad[kW3 + row], fmaf(V.b2[row], gd, d));
+        atomicAdd(&grad[kW3 + row], gd != 0.0f ? fmaf(V.b2[row], gd, d) : d);
       }
+    }
+    const uint4 left = *reinterpret_cast<const uint4 *>(bad);
+    if (left.x | left.y | left.z | left.w) {
+      __syncthreads();   // (part has been read)
+      for (uint32_t r = 0; r < kTileS; ++r)
+        if ((bad[r >> 5] >> (r & 31u)) & 1u) add_sample(sm, V, part, r, bad_dy[r], grad);
+      if (threadIdx.x < 4) bad[threadIdx.x] = 0;
     }
     store_x<kGradThreads>(sm + GradSmem::x, xr);
     fence_proxy_async_smem();
