@@ -375,6 +375,14 @@ esc_status esc_selftest_wait_timeout(uint64_t limit_ns, void *stream);
  * rows per unit, the number of units, and the reciprocal that maps a group
  * to its unit (ceil(2^32 / groups per unit), 0 for one group). */
 esc_status esc_debug_fail_allocs(int32_t n);
+/* esc_debug_taint_slot(when): the next synchronous sub-query call that
+ * reports through a call slot (esc_selectivity, esc_bitmap_build) finds an
+ * expired wait's marks in the slot's launch header, as a warp of a launch
+ * that gave up leaves them: 1, before its own launch, so that the blocks
+ * leave early; 2, after its launch, which then counts as expired.  Either
+ * way that call returns ESC_ETIMEOUT, and later calls are not affected.
+ * 0 turns it off. */
+esc_status esc_debug_taint_slot(int32_t when);
 esc_status esc_build_checked(int32_t *flag);
 esc_status esc_debug_write_units(uint64_t nrows, int32_t slots, uint32_t *out);
 

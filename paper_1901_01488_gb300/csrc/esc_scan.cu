@@ -408,7 +408,7 @@ struct StageMeta {
   int32_t q;       // query index, -1 = end of work
   uint32_t tile;   // tile index within the query
   uint32_t rows;   // valid rows in this tile
-  uint32_t dead;   // 1: the launch is aborting, skip the work (same for every reader)
+  uint32_t dead;   // with q -1: the launch is aborting, work is left
   uint32_t pad[4];
 };
 
@@ -575,6 +575,7 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
       if (u >= L.total_units || dead) {
         if (mbar_wait(&empty_bar[s], phase ^ 1u, hdr, kWaitLimitNs, true) && lane == 0) {
           meta[s].q = -1;
+          meta[s].dead = dead;
           mbar_arrive(&full_bar[s]);
         }
         break;
@@ -635,7 +636,6 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
           m.q = qc;
           m.tile = tile;
           m.rows = rows;
-          m.dead = dead;
           mbar_arrive_expect_tx(&full_bar[s], tot);
         }
         __syncwarp();
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
     const bool got = mbar_wait(&full_bar[s], phase, hdr);
     const StageMeta mt = meta[s];
     const bool end = !got || mt.q < 0;
-    if (lane == 0 && (!got || mt.dead != 0)) block_sum[2] = 1;
+    if (lane == 0 && end && (!got || mt.dead != 0)) block_sum[2] = 1;
     const Query *Q = &qslot[single ? 0 : s];
     if (uacc_ptr && end) {
       const uint32_t t = __reduce_add_sync(FULL, uacc);
@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
       if (lane == 0) j = (int)atomicAdd(&take[s], 1u);
       return __shfl_sync(FULL, j, 0);
     };
-    if (mt.dead == 0 && stage_in_bounds(Q, ngroups, hdr, lane)) {
+    if (stage_in_bounds(Q, ngroups, hdr, lane)) {
       // one evaluation loop for every mode (a single inlined copy of the
       // interpreter); the per-group epilogue branches on the mode (uniform)
       const uint32_t nwords = (Q->nrows + 31u) / 32u;
@@ -1332,7 +1332,6 @@ __global__ void __launch_bounds__(kThreads, 1) shared_kernel(const __grid_consta
           m.q = 0;
           m.tile = tile;
           m.rows = rows;
-          m.dead = dead;
           mbar_arrive_expect_tx(&full_bar[s], tot);
         }
         __syncwarp();
@@ -1355,31 +1354,29 @@ __global__ void __launch_bounds__(kThreads, 1) shared_kernel(const __grid_consta
     const bool got = mbar_wait(&full_bar[s], phase, hdr);
     const StageMeta mt = meta[s];
     if (!got || mt.q < 0) break;
-    if (mt.dead == 0) {
-      const uint8_t *stage = stages + (size_t)s * kStageBytes;
-      const uint32_t rows = mt.rows;
-      const int ngroups = (int)((rows + kGroup - 1) / kGroup);
-      const int npairs = (ngroups + 1) >> 1;
-      const int items = npairs * nq;
-      for (;;) {
-        int j = 0;
-        if (lane == 0) j = (int)atomicAdd(&take[s], 1u);
-        j = __shfl_sync(FULL, j, 0);
-        if (j >= items) break;
-        const int qi = j / npairs;
-        const int g = 2 * (j - qi * npairs), g1 = g + 1;
-        if (qi != acc_q) {
-          const uint32_t t = __reduce_add_sync(FULL, acc);
-          if (lane == 0 && t) atomicAdd(&cnt[acc_q], t);
-          acc = 0;
-          acc_q = qi;
-        }
-        const int gs[2] = {g, g1 < ngroups ? g1 : g};
-        uint32_t mm[2];
-        eval_groups<2, true>(&L.queries[qi], stage, gs, lane, mm);
-        acc += __popc(mm[0] & valid_mask(g, lane, rows));
-        if (g1 < ngroups) acc += __popc(mm[1] & valid_mask(g1, lane, rows));
+    const uint8_t *stage = stages + (size_t)s * kStageBytes;
+    const uint32_t rows = mt.rows;
+    const int ngroups = (int)((rows + kGroup - 1) / kGroup);
+    const int npairs = (ngroups + 1) >> 1;
+    const int items = npairs * nq;
+    for (;;) {
+      int j = 0;
+      if (lane == 0) j = (int)atomicAdd(&take[s], 1u);
+      j = __shfl_sync(FULL, j, 0);
+      if (j >= items) break;
+      const int qi = j / npairs;
+      const int g = 2 * (j - qi * npairs), g1 = g + 1;
+      if (qi != acc_q) {
+        const uint32_t t = __reduce_add_sync(FULL, acc);
+        if (lane == 0 && t) atomicAdd(&cnt[acc_q], t);
+        acc = 0;
+        acc_q = qi;
       }
+      const int gs[2] = {g, g1 < ngroups ? g1 : g};
+      uint32_t mm[2];
+      eval_groups<2, true>(&L.queries[qi], stage, gs, lane, mm);
+      acc += __popc(mm[0] & valid_mask(g, lane, rows));
+      if (g1 < ngroups) acc += __popc(mm[1] & valid_mask(g1, lane, rows));
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty_bar[s]);
@@ -1997,6 +1994,23 @@ esc_status run_single(const esc_table *t, const esc_pred *p, esc_rows *rows, int
   return ESC_OK;
 }
 
+// Test hook (esc_debug_taint_slot): the marks of an expired wait in a slot's header.
+static std::atomic<int32_t> g_taint_slot{0};
+static cudaError_t taint_slot(const SlotRef &s, cudaStream_t st) {
+  ScratchHdr h{};
+  h.status = ESC_ETIMEOUT;
+  h.abort = 1;
+  cudaError_t e = cudaMemcpyAsync(&s.dev->hdr, &h, sizeof h, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
+// Makes a slot whose launch gave up usable again: warps that were still waiting
+// when it reported may have raised the abort flag or taken a ticket since.
+static bool reset_slot(const SlotRef &s, cudaStream_t st) {
+  return cudaStreamSynchronize(st) == cudaSuccess && cudaMemsetAsync(s.dev, 0, sizeof *s.dev, st) == cudaSuccess &&
+         cudaStreamSynchronize(st) == cudaSuccess;
+}
+
 // A synchronous sub-query: in a call slot where one is free, else as an
 // asynchronous one whose count and status are copied back.  The slot saves the
 // allocation, the memset and the copy: a count of a 10,000-row table takes 19
@@ -2042,7 +2056,9 @@ esc_status run_sync(const esc_table *t, const esc_pred *p, esc_rows *rows, int m
       return s;
     }
   }
-  s = launch_scan(L, query_shape(L.q0, p->tuning), st, mem != nullptr);
+  const int32_t taint = g_taint_slot.load(std::memory_order_relaxed) ? g_taint_slot.exchange(0) : 0;
+  if (taint == 1) ESC_CK(taint_slot(slot, st));
+  s = launch_scan(L, query_shape(L.q0, p->tuning), st, mem != nullptr && taint != 1);
   if (s == ESC_OK && mode == MODE_SELECT) s = launch_write(L, L.q0.nwunits, st);
   if (mem) cudaFreeAsync(mem, st);
   // (after a failure the slot stays taken: its launch may still be running)
@@ -2054,7 +2070,11 @@ esc_status run_sync(const esc_table *t, const esc_pred *p, esc_rows *rows, int m
   ScratchHdr h{};
   h.status = slot.host->status;
   const uint64_t c = slot.host->count;
-  give_slot(slot);
+  if (taint == 2) {
+    ESC_CK(taint_slot(slot, st));
+    h.status = ESC_ETIMEOUT;
+  }
+  if (h.status == 0 || reset_slot(slot, st)) give_slot(slot);
   if (h.status != 0) return device_status(h, "sub-query");
   *count = c;
   return ESC_OK;
@@ -2090,6 +2110,13 @@ esc_status esc_selectivity(const esc_table *t, const esc_pred *p, uint64_t *coun
     rows->written = std::min<uint64_t>(c, rows->capacity);
     if (c > rows->capacity) return fail(ESC_ETRUNC, "esc_selectivity: more qualifying rows than capacity");
   }
+  clear_error();
+  return ESC_OK;
+}
+
+esc_status esc_debug_taint_slot(int32_t when) {
+  if (when < 0 || when > 2) return fail(ESC_EINVAL, "esc_debug_taint_slot: when must be 0, 1 or 2");
+  g_taint_slot.store(when);
   clear_error();
   return ESC_OK;
 }

@@ -87,6 +87,7 @@ _sig = {
     "esc_selectivity_batch_async": ([ctypes.POINTER(_P), ctypes.POINTER(_P), ctypes.c_int32,
                                      ctypes.POINTER(esc_rows), _P, _P, _P], _S),
     "esc_debug_fail_allocs": ([ctypes.c_int32], _S),
+    "esc_debug_taint_slot": ([ctypes.c_int32], _S),
     "esc_debug_write_units": ([ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32)], _S),
     "esc_build_checked": ([ctypes.POINTER(ctypes.c_int32)], _S),
     "esc_mlp_forward": ([_P, ctypes.c_uint64, _P, _P, _P, _P], _S),
@@ -387,6 +388,12 @@ def esc_mlp_adam(params: torch.Tensor, w_bf16: torch.Tensor, grad: torch.Tensor,
 
 def esc_debug_fail_allocs(n: int) -> None:
     _check(_lib.esc_debug_fail_allocs(n), "esc_debug_fail_allocs")
+
+
+def esc_debug_taint_slot(when: int) -> None:
+    """The next synchronous sub-query finds an expired wait's marks in its
+    call slot: 1 before its launch, 2 after it; 0 turns it off."""
+    _check(_lib.esc_debug_taint_slot(when), "esc_debug_taint_slot")
 
 
 def esc_debug_write_units(nrows: int, slots: int) -> Tuple[int, int, int]:
