@@ -904,7 +904,9 @@ __device__ __forceinline__ void flush_sparse(const GatherInfo &G, const uint32_t
         const uint32_t e = ent[t];
         row[k] = row_ref + (e >> 16);
         pos[k] = pos_ref + (e & 0xffffu);
-        if (pos[k] < cap && ESC_INB(hdr, row[k] < G.nrows, 22, row[k])) ok |= 1u << k;
+        // (a scan that gave up leaves bitmap words unwritten: whatever they
+        // hold, no row past the table is read)
+        if (pos[k] < cap && ESC_INB(hdr, row[k] < G.nrows, 22, row[k]) && row[k] < G.nrows) ok |= 1u << k;
       }
     }
 #pragma unroll

@@ -65,3 +65,28 @@ def test_hook_is_off_by_default(world):
     esc.esc_debug_taint_slot(1)
     esc.esc_debug_taint_slot(0)
     check("count", call(esc, tbl, "count", len(ids)), ids, vals)
+
+
+def test_materialising_after_an_expired_scan(world):
+    """The write pass over a bitmap that the scan did not finish (what its
+    memory held before is there instead): no row past the table, nothing
+    past the buffers."""
+    esc, tbl, ids, vals = world
+    rows = ROWS // 256 * 256 + 10                    # the last group's other rows are set in what memory holds
+    small = datagen.skewed_table(rows, seed=32, device="cuda")
+    stbl = esc.Table.from_datagen(small)
+    p, every = esc.Predicate(stbl, TEXT, ("price",)), esc.Predicate(tbl, "day >= 0 AND code25 < 200", ())
+    for _ in range(4):
+        out = every.alloc_rows(ROWS)
+        esc.esc_selectivity(tbl.handle, every.handle, out)
+        got = torch.zeros(rows + 64, dtype=torch.int32, device="cuda")
+        col = torch.full((rows + 64,), -7, dtype=torch.int64, device="cuda")
+        got[rows:] = -7
+        esc.esc_debug_taint_slot(1)
+        with pytest.raises(esc.EscError) as ei:
+            esc.esc_selectivity(stbl.handle, p.handle, (rows, got, [col]))
+        assert ei.value.status == esc.ESC_ETIMEOUT
+        torch.cuda.synchronize()
+        assert bool((got[:rows] >= 0).all()) and int(got[:rows].max()) < rows
+        assert bool((got[rows:] == -7).all()) and bool((col[rows:] == -7).all())
+    check("select", call(esc, tbl, "select", len(ids)), ids, vals)
