@@ -314,7 +314,8 @@ esc_status esc_semijoin_counts(const esc_table *fact, const char *const *fk_cols
  * is synchronised. */
 #define ESC_MLP_PARAMS 24961
 
-/* y[i] = network(x[i]) for `batch` rows of 64 bfloat16 features. */
+/* y[i] = network(x[i]) for `batch` rows of 64 bfloat16 features.  Where a
+ * wait for the tensor cores gives up (after 2 s), y is NaN. */
 esc_status esc_mlp_forward(const uint16_t *x_bf16, uint64_t batch, const uint16_t *w_bf16,
                            const float *params, float *y, void *stream);
 
@@ -322,7 +323,8 @@ esc_status esc_mlp_forward(const uint16_t *x_bf16, uint64_t batch, const uint16_
  * over the batch, and to *loss_sum the sum of squared errors.  The caller
  * zeroes both beforehand.  A sample with an infinite or NaN residual makes
  * non-finite only the entries it contributes to: a unit it leaves inactive
- * gets nothing from it. */
+ * gets nothing from it.  When a wait for the tensor cores gives up (after
+ * 2 s), *loss_sum becomes NaN: grad is then incomplete and not to be used. */
 esc_status esc_mlp_grad(const uint16_t *x_bf16, const float *target, uint64_t batch,
                         const uint16_t *w_bf16, const float *params, float *grad, float *loss_sum,
                         void *stream);
@@ -383,6 +385,10 @@ esc_status esc_debug_fail_allocs(int32_t n);
  * way that call returns ESC_ETIMEOUT, and later calls are not affected.
  * 0 turns it off. */
 esc_status esc_debug_taint_slot(int32_t when);
+/* esc_debug_mlp_give_up(wait): in the checked build, the wait of this number
+ * (from 1) of every block of the following MLP kernels gives up, as if its
+ * limit had passed; 0 turns it off.  ESC_EINVAL in the release build. */
+esc_status esc_debug_mlp_give_up(uint32_t wait);
 esc_status esc_build_checked(int32_t *flag);
 esc_status esc_debug_write_units(uint64_t nrows, int32_t slots, uint32_t *out);
 
