@@ -389,6 +389,10 @@ esc_status esc_debug_taint_slot(int32_t when);
  * (from 1) of every block of the following MLP kernels gives up, as if its
  * limit had passed; 0 turns it off.  ESC_EINVAL in the release build. */
 esc_status esc_debug_mlp_give_up(uint32_t wait);
+/* esc_debug_shrink_table(chunks): in the checked build, shared scans by table
+ * lookup take their table to be this many 16-byte chunks shorter than it is, so
+ * that its checks fire; 0 turns it off.  ESC_EINVAL in the release build. */
+esc_status esc_debug_shrink_table(uint32_t chunks);
 esc_status esc_build_checked(int32_t *flag);
 esc_status esc_debug_write_units(uint64_t nrows, int32_t slots, uint32_t *out);
 

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -69,7 +70,7 @@ struct Operand {
   int32_t da, db;         // their esc_dtype
   int32_t kind;           // OperandKind of the value searched
   uint32_t ncuts;         // intervals: ncuts + 1
-  uint32_t steps;         // binary-search steps; 2^steps - 1 padded cuts
+  uint32_t steps;         // binary-search steps; 2^steps - 1 padded cuts at least
   uint32_t cut_off;       // byte offset of the cuts
   uint32_t table_off;     // byte offset of interval 0's bit row
   // buckets of equal width (2^shift) over the cuts' values (kind OPD_32; bsteps ~0: none)
@@ -81,6 +82,10 @@ struct Operand {
   uint32_t K;
   int32_t sh1, sh2;
   uint64_t d, M, mult;
+#ifdef ESC_CHECKED
+  uint32_t padded;        // cuts with their padding
+  uint32_t nbuckets;
+#endif
 };
 
 struct StageColumn {
@@ -121,6 +126,10 @@ struct BuildArgs {
   const uint2 *box_ref;       // its range of refs
   const int64_t *pool;
 };
+
+[[maybe_unused]] __device__ __forceinline__ uint32_t width_of(int32_t dt) {
+  return dt == ESC_U8 ? 1u : dt == ESC_U16 ? 2u : dt == ESC_I32 ? 4u : 8u;
+}
 
 __device__ __forceinline__ int64_t load_value(const uint8_t *p, int32_t dt, uint32_t row) {
   switch (dt) {
@@ -179,7 +188,8 @@ struct SortJob {
   uint32_t wide;      // 64-bit cuts
 };
 constexpr uint32_t kSortCuts = 64;   // cuts per block
-__global__ void __launch_bounds__(1024) sort_cuts_kernel(const int64_t *unsorted, const SortJob *jobs, uint8_t *cuts) {
+__global__ void __launch_bounds__(1024) sort_cuts_kernel(const int64_t *unsorted, const SortJob *jobs, uint8_t *cuts,
+                                                         [[maybe_unused]] ScratchHdr *hdr) {
   __shared__ uint32_t rank[kSortCuts];
   const SortJob J = jobs[blockIdx.y];
   if (blockIdx.x * kSortCuts >= J.padded) return;   // uniform
@@ -202,15 +212,18 @@ __global__ void __launch_bounds__(1024) sort_cuts_kernel(const int64_t *unsorted
   if (part != 0 || i >= J.padded) return;
   // padding past the last cut: the type's largest value
   const uint32_t at = i < J.n ? rank[threadIdx.x] : i;
+  if (!ESC_INB(hdr, at < J.padded, 48, at)) return;
   if (J.wide) reinterpret_cast<int64_t *>(cuts + J.dst_off)[at] = i < J.n ? v : INT64_MAX;
   else reinterpret_cast<int32_t *>(cuts + J.dst_off)[at] = i < J.n ? (int32_t)v : INT32_MAX;
 }
 
 // Number of an operand's sorted cuts <= v (its interval of value v).
-__device__ __forceinline__ uint32_t interval_of(const Operand &o, const uint8_t *cuts, int64_t v) {
+__device__ __forceinline__ uint32_t interval_of(const BoxLaunch &L, const Operand &o, int64_t v) {
+  const uint8_t *cuts = L.cuts;
   if (o.kind == OPD_U8) return v < 0 ? 0u : (uint32_t)min(v, (int64_t)255);
   uint32_t pos = 0;
   for (uint32_t h = 1u << o.steps >> 1; h; h >>= 1) {
+    if (!ESC_INB(L.hdr, pos + h <= o.padded, 44, pos + h)) return 0;
     const int64_t c = o.kind == OPD_64 ? reinterpret_cast<const int64_t *>(cuts + o.cut_off)[pos + h - 1]
                                        : (int64_t)reinterpret_cast<const int32_t *>(cuts + o.cut_off)[pos + h - 1];
     pos += c <= v ? h : 0u;
@@ -246,8 +259,8 @@ __global__ void __launch_bounds__(256) build_kernel(const __grid_constant__ BoxL
     const BoxTest &t = B.tests[B.refs[r0] >> 1];
     neg = B.refs[r0] & 1u;
     if (t.op == OP_RANGE) {
-      a = interval_of(o, L.cuts, t.lo);
-      len = interval_of(o, L.cuts, t.hi) - a + 1u;
+      a = interval_of(L, o, t.lo);
+      len = interval_of(L, o, t.hi) - a + 1u;
     } else {
       general = true;
     }
@@ -290,19 +303,20 @@ __global__ void __launch_bounds__(256) build_kernel(const __grid_constant__ BoxL
 
 // Numbers of sorted cuts <= v[k]: `steps` halvings of a padded array.
 template <typename T, int R>
-__device__ __forceinline__ void search(const uint8_t *cuts, uint32_t steps, uint32_t ncuts, const T (&v)[R], uint32_t (&pos)[R]) {
-  const T *cut = reinterpret_cast<const T *>(cuts) - 1;
+__device__ __forceinline__ void search([[maybe_unused]] const BoxLaunch &L, const Operand &o, const uint8_t *cuts,
+                                       const T (&v)[R], uint32_t (&pos)[R]) {
+  const T *cut = reinterpret_cast<const T *>(cuts + o.cut_off) - 1;
 #pragma unroll
   for (int k = 0; k < R; ++k) pos[k] = 0;
-  for (uint32_t h = 1u << steps >> 1; h; h >>= 1) {
+  for (uint32_t h = 1u << o.steps >> 1; h; h >>= 1) {
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const uint32_t t = pos[k] + h;
-      if (cut[t] <= v[k]) pos[k] = t;
+      if (ESC_INB(L.hdr, t <= o.padded, 44, t) && cut[t] <= v[k]) pos[k] = t;
     }
   }
 #pragma unroll
-  for (int k = 0; k < R; ++k) pos[k] = min(pos[k], ncuts);   // padding equals the largest value
+  for (int k = 0; k < R; ++k) pos[k] = min(pos[k], o.ncuts);   // padding equals the largest value
 }
 
 // The same with a table of buckets: the value's bucket gives the number of cuts
@@ -310,21 +324,22 @@ __device__ __forceinline__ void search(const uint8_t *cuts, uint32_t steps, uint
 // the bucket's own cuts, `bsteps` halvings for the fullest one.  Later buckets'
 // cuts lie above the value, so halvings past the bucket's end find nothing.
 template <int R>
-__device__ __forceinline__ void bucket_search(const Operand &o, const uint8_t *cuts, const uint8_t *buckets,
-                                              const int32_t (&v)[R], uint32_t (&pos)[R]) {
+__device__ __forceinline__ void bucket_search([[maybe_unused]] const BoxLaunch &L, const Operand &o,
+                                              const uint8_t *cuts, const uint8_t *buckets, const int32_t (&v)[R], uint32_t (&pos)[R]) {
   const int32_t *cut = reinterpret_cast<const int32_t *>(cuts + o.cut_off) - 1;
   const uint16_t *first = reinterpret_cast<const uint16_t *>(buckets + o.bucket_off);
   int32_t w[R];
 #pragma unroll
   for (int k = 0; k < R; ++k) {
     w[k] = max(o.base, min(v[k], o.top));
-    pos[k] = first[((uint32_t)w[k] - (uint32_t)o.base) >> o.shift];
+    const uint32_t b = ((uint32_t)w[k] - (uint32_t)o.base) >> o.shift;
+    pos[k] = ESC_INB(L.hdr, b < o.nbuckets, 43, b) ? first[b] : 0u;
   }
   for (uint32_t h = 1u << o.bsteps >> 1; h; h >>= 1) {
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const uint32_t t = pos[k] + h;
-      if (cut[t] <= w[k]) pos[k] = t;
+      if (ESC_INB(L.hdr, t <= o.padded, 44, t) && cut[t] <= w[k]) pos[k] = t;
     }
   }
 #pragma unroll
@@ -332,10 +347,10 @@ __device__ __forceinline__ void bucket_search(const Operand &o, const uint8_t *c
 }
 
 template <int R>
-__device__ __forceinline__ void search32(const Operand &o, const uint8_t *cuts, const uint8_t *buckets,
-                                         const int32_t (&v)[R], uint32_t (&pos)[R]) {
-  if (o.bsteps != ~0u) bucket_search<R>(o, cuts, buckets, v, pos);
-  else search<int32_t, R>(cuts + o.cut_off, o.steps, o.ncuts, v, pos);
+__device__ __forceinline__ void search32(const BoxLaunch &L, const Operand &o, const uint8_t *cuts,
+                                         const uint8_t *buckets, const int32_t (&v)[R], uint32_t (&pos)[R]) {
+  if (o.bsteps != ~0u) bucket_search<R>(L, o, cuts, buckets, v, pos);
+  else search<int32_t, R>(L, o, cuts, v, pos);
 }
 
 __device__ __forceinline__ int32_t saturate32(int64_t v) {
@@ -344,9 +359,17 @@ __device__ __forceinline__ int32_t saturate32(int64_t v) {
 
 // The intervals of operand o of R rows of a staged tile: rows row + k * kBoxThreads.
 template <int R>
-__device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage, const uint8_t *cuts, const uint8_t *buckets,
-                                          uint32_t row, uint32_t (&pos)[R]) {
+__device__ __forceinline__ void intervals(const BoxLaunch &L, const Operand &o, const uint8_t *stage, const uint8_t *cuts,
+                                          const uint8_t *buckets, uint32_t row, uint32_t (&pos)[R]) {
   const uint8_t *a = stage + o.a;
+#ifdef ESC_CHECKED
+  const uint32_t rows = row + (R - 1) * kBoxThreads + 1;
+  if (!ESC_INB(L.hdr, o.a + rows * width_of(o.da) <= L.stage_bytes, 45, o.a) ||
+      (o.b != ~0u && !ESC_INB(L.hdr, o.b + rows * width_of(o.db) <= L.stage_bytes, 45, o.b))) {
+    for (int k = 0; k < R; ++k) pos[k] = 0;
+    return;
+  }
+#endif
   if (o.kind == OPD_U8) {
 #pragma unroll
     for (int k = 0; k < R; ++k) pos[k] = a[row + k * kBoxThreads];
@@ -361,7 +384,7 @@ __device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage
 #pragma unroll
       for (int k = 0; k < R; ++k) v[k] = reinterpret_cast<const uint16_t *>(a)[row + k * kBoxThreads];
     }
-    search32<R>(o, cuts, buckets, v, pos);
+    search32<R>(L, o, cuts, buckets, v, pos);
     return;
   }
   long long v[R];
@@ -372,12 +395,12 @@ __device__ __forceinline__ void intervals(const Operand &o, const uint8_t *stage
     for (int k = 0; k < R; ++k) v[k] = udf_value(o, v[k], load_value(stage + o.b, o.db, row + k * kBoxThreads));
   }
   if (o.kind == OPD_64) {
-    search<long long, R>(cuts + o.cut_off, o.steps, o.ncuts, v, pos);
+    search<long long, R>(L, o, cuts, v, pos);
   } else {
     int32_t w[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) w[k] = saturate32(v[k]);
-    search32<R>(o, cuts, buckets, w, pos);
+    search32<R>(L, o, cuts, buckets, w, pos);
   }
 }
 
@@ -556,7 +579,7 @@ __global__ void __launch_bounds__(kBoxThreads, VEC == 4 ? 2 : 3) box_rows_kernel
     for (int c = 0; c < L.nop; ++c) {
       const Operand &o = L.op[c];
       uint32_t pos[kRows];
-      intervals<kRows>(o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
+      intervals<kRows>(L, o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
 #pragma unroll
       for (int k = 0; k < kRows; ++k) {
         uint32_t off = o.table_off + pos[k] * (4u * VEC);
@@ -624,7 +647,8 @@ __global__ void __launch_bounds__(kBoxThreads, 2) box_words_kernel(const __grid_
       if (live) flush_planes<4>(p, cnt, word0, L.nboxes, lane);
       pending = 0;
       word0 = (j / ring.mine * lanes + sub) * 4;
-      live = word0 * 4u < L.stride;   // a bit row may be shorter than the chunk
+      live = word0 * 4u < L.stride &&   // a bit row may be shorter than the chunk
+             ESC_INB(L.hdr, word0 / 4 < (L.nboxes + 127) / 128, 47, word0);
       lane_off = live ? word0 * 4u : 0u;
       need = live ? L.lane_ops[word0 / 4] : 0u;
     }
@@ -635,7 +659,7 @@ __global__ void __launch_bounds__(kBoxThreads, 2) box_words_kernel(const __grid_
     for (int c = 0; c < L.nop; ++c) {
       const Operand &o = L.op[c];
       uint32_t pos[2];
-      intervals<2>(o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
+      intervals<2>(L, o, stage, cuts, sm + L.smem_bucket, threadIdx.x, pos);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         uint32_t off = o.table_off + pos[k] * L.stride;
@@ -660,7 +684,7 @@ __global__ void __launch_bounds__(kBoxThreads, 2) box_words_kernel(const __grid_
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           const uint32_t r = (warp * steps + q + u + k) * rows_per_step + rsub;
-          const bool in = live && q + u + k < steps && r < rows;
+          const bool in = live && q + u + k < steps && r < rows && ESC_INB(L.hdr, r < (uint32_t)kTile, 46, r);
           ro[k] = &offs[(in ? r : 0u) * nopp];
 #pragma unroll
           for (int v = 0; v < 4; ++v) x[k].w[v] = in ? FULL : 0u;
@@ -824,7 +848,11 @@ uint32_t round16(uint64_t b) { return (uint32_t)((b + 15) & ~(uint64_t)15); }
 
 }  // namespace
 
-// Everything a pass needs on the host; built by plan_boxes.
+#ifdef ESC_CHECKED
+std::atomic<uint32_t> g_shrink_table{0};   // esc_debug_shrink_table
+#endif
+
+// What a pass needs on the host; add_predicate adds to it.
 struct BoxPlan {
   std::vector<HostOperand> ops;
   std::vector<BoxTest> tests;
@@ -963,6 +991,9 @@ void make_buckets(Operand &o, const std::vector<int64_t> &cuts, uint32_t most, s
   o.top = (int32_t)top;
   o.shift = shift;
   o.bucket_off = (uint32_t)(out.size() * 2);
+#ifdef ESC_CHECKED
+  o.nbuckets = n;
+#endif
   for (uint32_t k = 0; k < n; ++k) out.push_back((uint16_t)before[shift ? k : k + 1]);
 }
 
@@ -1082,6 +1113,9 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
     const uint32_t padded = std::max((1u << o.steps) - 1, o.bsteps == ~0u ? 0u : o.ncuts + (1u << o.bsteps) - 1);
     const uint32_t w = o.kind == OPD_64 ? 8u : 4u;
     padded_cuts[c] = padded;
+#ifdef ESC_CHECKED
+    o.padded = padded;
+#endif
     o.cut_off = (uint32_t)cut_bytes;
     if (job) {
       job->padded = padded;
@@ -1209,7 +1243,8 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
     uint32_t most = 0;
     for (auto &j : jobs) most = std::max(most, j.padded);
     sort_cuts_kernel<<<dim3((most + kSortCuts - 1) / kSortCuts, (unsigned)jobs.size()), 1024, 0, st>>>(
-        reinterpret_cast<const int64_t *>(dev + a_uns), reinterpret_cast<const SortJob *>(dev + a_jobs), dev + a_cuts);
+        reinterpret_cast<const int64_t *>(dev + a_uns), reinterpret_cast<const SortJob *>(dev + a_jobs), dev + a_cuts,
+        hdr);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -1222,6 +1257,9 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
   }
   if (e == cudaSuccess) {
     if (by_row) L.table_bytes = round16(table_bytes);   // what the kernel copies
+#ifdef ESC_CHECKED
+    L.table_bytes -= std::min(g_shrink_table.load(), L.table_bytes / 16) * 16;
+#endif
     const uint32_t fit = std::max<uint32_t>(1, (227u * 1024) / (smem + 1024));
     const uint32_t ctas = std::min<uint32_t>(fit, vec == 4 ? 2 : 3);
     const uint32_t grid = std::min<uint32_t>((uint32_t)sms * ctas, (L.nrows + L.tile - 1) / L.tile);
@@ -1240,3 +1278,14 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
 }
 
 }  // namespace esc
+
+extern "C" esc_status esc_debug_shrink_table(uint32_t chunks) {
+#ifdef ESC_CHECKED
+  esc::g_shrink_table.store(chunks);
+  esc::clear_error();
+  return ESC_OK;
+#else
+  (void)chunks;
+  return esc::fail(ESC_EINVAL, "esc_debug_shrink_table: only in the checked build");
+#endif
+}

@@ -1315,6 +1315,9 @@ __global__ void __launch_bounds__(kThreads, 1) shared_kernel(const __grid_consta
           tail = bytes - bulk;
           src = Y.ref_ptr[lane] + (size_t)r0 * w;
           dst = stage + Y.stage_off[lane];
+          if (!ESC_INB(hdr, Y.stage_off[lane] + bytes <= kStageBytes, 1, Y.stage_off[lane] + bytes) ||
+              !ESC_INB(hdr, (uint64_t)r0 + rows <= Y.nrows, 2, r0 + rows))
+            bulk = tail = 0;
         }
         if (__ballot_sync(FULL, tail != 0)) {
           for (int c = 0; c < nref; ++c) {
@@ -1374,6 +1377,7 @@ __global__ void __launch_bounds__(kThreads, 1) shared_kernel(const __grid_consta
         acc = 0;
         acc_q = qi;
       }
+      if (!stage_in_bounds(&L.queries[qi], ngroups, hdr, lane)) continue;
       const int gs[2] = {g, g1 < ngroups ? g1 : g};
       uint32_t mm[2];
       eval_groups<2, true>(&L.queries[qi], stage, gs, lane, mm);
@@ -2646,6 +2650,16 @@ static esc_status run_shared_group(const esc_table *t, const esc_pred *const *pr
     }
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(dev_counts, counts, (size_t)n * 8, cudaMemcpyDeviceToDevice, st);
+#ifdef ESC_CHECKED   // the checked kernels' findings: this build's call waits for them
+  ScratchHdr found{};
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    e = cudaMemcpyAsync(&found, hdr, sizeof found, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && found.status != 0) return device_status(found, "esc_selectivity_shared_async");
+  }
+#endif
   if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_selectivity_shared_async: ") + cudaGetErrorString(e));
   return ESC_OK;
 }

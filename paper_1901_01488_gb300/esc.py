@@ -89,6 +89,7 @@ _sig = {
     "esc_debug_fail_allocs": ([ctypes.c_int32], _S),
     "esc_debug_taint_slot": ([ctypes.c_int32], _S),
     "esc_debug_mlp_give_up": ([ctypes.c_uint32], _S),
+    "esc_debug_shrink_table": ([ctypes.c_uint32], _S),
     "esc_debug_write_units": ([ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32)], _S),
     "esc_build_checked": ([ctypes.POINTER(ctypes.c_int32)], _S),
     "esc_mlp_forward": ([_P, ctypes.c_uint64, _P, _P, _P, _P], _S),
@@ -400,6 +401,11 @@ def esc_debug_taint_slot(when: int) -> None:
 def esc_debug_mlp_give_up(wait: int) -> None:
     """Checked build: the MLP kernels' wait of this number in every block gives up; 0 turns it off."""
     _check(_lib.esc_debug_mlp_give_up(wait), "esc_debug_mlp_give_up")
+
+
+def esc_debug_shrink_table(chunks: int) -> None:
+    """Checked build: lookup tables are taken to be this many 16-byte chunks shorter; 0 turns it off."""
+    _check(_lib.esc_debug_shrink_table(chunks), "esc_debug_shrink_table")
 
 
 def esc_debug_write_units(nrows: int, slots: int) -> Tuple[int, int, int]:
