@@ -377,6 +377,9 @@ esc_status esc_selftest_wait_timeout(uint64_t limit_ns, void *stream);
  * rows per unit, the number of units, and the reciprocal that maps a group
  * to its unit (ceil(2^32 / groups per unit), 0 for one group). */
 esc_status esc_debug_fail_allocs(int32_t n);
+/* esc_debug_fail_host_allocs(n): the same for the next n arrays that
+ * asynchronous batches and shared scans stage in host memory. */
+esc_status esc_debug_fail_host_allocs(int32_t n);
 /* esc_debug_taint_slot(when): the next synchronous sub-query call that
  * reports through a call slot (esc_selectivity, esc_bitmap_build) finds an
  * expired wait's marks in the slot's launch header, as a warp of a launch

@@ -1196,11 +1196,11 @@ esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long
                  a_uns = place(unsorted.size() * 8 + 8), a_buckets = place(buckets.size() * 2 + 16),
                  a_cuts = place(L.cut_bytes + 16), upload = at,
                  a_table = place(round16(table_bytes));
+  HostStage stage(upload, st);   // (throws without host memory: before there is device memory to give back)
   void *mem = nullptr;
   esc_status s = alloc_async(&mem, at, st);
   if (s != ESC_OK) return s;
   uint8_t *dev = static_cast<uint8_t *>(mem);
-  HostStage stage(upload, st);
   uint8_t *h = stage.data();
   auto put = [&](uint64_t a, const void *src, size_t bytes) {
     if (bytes) std::memcpy(h + a, src, bytes);

@@ -803,14 +803,16 @@ void fill_query_program(const esc_pred *p, Query *q) {
   q->npool = (uint32_t)p->pool.size();
 }
 
-std::atomic<int32_t> g_fail_allocs{0};
+std::atomic<int32_t> g_fail_allocs{0}, g_fail_host_allocs{0};
 
-bool inject_alloc_failure() {
-  int32_t n = g_fail_allocs.load();
-  while (n > 0 && !g_fail_allocs.compare_exchange_weak(n, n - 1)) {
+static bool count_down(std::atomic<int32_t> &left) {
+  int32_t n = left.load();
+  while (n > 0 && !left.compare_exchange_weak(n, n - 1)) {
   }
   return n > 0;
 }
+bool inject_alloc_failure() { return count_down(g_fail_allocs); }
+bool inject_host_failure() { return count_down(g_fail_host_allocs); }
 
 esc_status device_status(const ScratchHdr &h, const char *where) {
   if (h.status == (unsigned)ESC_EBOUNDS)
@@ -844,6 +846,13 @@ const char *esc_status_string(esc_status s) {
     case ESC_EBOUNDS: return "ESC_EBOUNDS";
   }
   return "ESC_UNKNOWN";
+}
+
+esc_status esc_debug_fail_host_allocs(int32_t n) {
+  if (n < 0) return fail(ESC_EINVAL, "esc_debug_fail_host_allocs: n must be >= 0");
+  g_fail_host_allocs.store(n);
+  clear_error();
+  return ESC_OK;
 }
 
 esc_status esc_debug_fail_allocs(int32_t n) {

@@ -236,6 +236,7 @@ esc_status device_status(const ScratchHdr &h, const char *where);
 // Test hook: true when a device allocation of the library is to fail
 // (esc_debug_fail_allocs counts them down).
 bool inject_alloc_failure();
+bool inject_host_failure();   // the same for host staging memory (esc_debug_fail_host_allocs)
 // A free slot of the current device for one synchronous call on `stream`
 // (esc_scan.cu): null when all are in use or the stream is being captured; the
 // call then allocates scratch.  give_slot returns it when the launch is known

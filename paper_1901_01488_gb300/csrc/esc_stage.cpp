@@ -2,6 +2,9 @@
 #include "esc_stage.h"
 
 #include <mutex>
+#include <new>
+
+#include "esc_internal.h"
 
 namespace esc {
 
@@ -64,7 +67,9 @@ StageBlock *acquire(size_t bytes, cudaStream_t st) {
 
 }  // namespace
 
-HostStage::HostStage(size_t bytes, cudaStream_t st) : bytes_(bytes), st_(st), block_(acquire(bytes, st)) {
+HostStage::HostStage(size_t bytes, cudaStream_t st) : bytes_(bytes), st_(st) {
+  if (inject_host_failure()) throw std::bad_alloc();
+  block_ = acquire(bytes, st);
   if (!block_) own_.reset(new uint8_t[bytes ? bytes : 1]);
   data_ = block_ ? block_->mem : own_.get();
 }

@@ -90,6 +90,7 @@ _sig = {
     "esc_debug_taint_slot": ([ctypes.c_int32], _S),
     "esc_debug_mlp_give_up": ([ctypes.c_uint32], _S),
     "esc_debug_shrink_table": ([ctypes.c_uint32], _S),
+    "esc_debug_fail_host_allocs": ([ctypes.c_int32], _S),
     "esc_debug_write_units": ([ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32)], _S),
     "esc_build_checked": ([ctypes.POINTER(ctypes.c_int32)], _S),
     "esc_mlp_forward": ([_P, ctypes.c_uint64, _P, _P, _P, _P], _S),
@@ -406,6 +407,10 @@ def esc_debug_mlp_give_up(wait: int) -> None:
 def esc_debug_shrink_table(chunks: int) -> None:
     """Checked build: lookup tables are taken to be this many 16-byte chunks shorter; 0 turns it off."""
     _check(_lib.esc_debug_shrink_table(chunks), "esc_debug_shrink_table")
+
+
+def esc_debug_fail_host_allocs(n: int) -> None:
+    _check(_lib.esc_debug_fail_host_allocs(n), "esc_debug_fail_host_allocs")
 
 
 def esc_debug_write_units(nrows: int, slots: int) -> Tuple[int, int, int]:
