@@ -388,6 +388,10 @@ esc_status esc_debug_fail_host_allocs(int32_t n);
  * way that call returns ESC_ETIMEOUT, and later calls are not affected.
  * 0 turns it off. */
 esc_status esc_debug_taint_slot(int32_t when);
+/* esc_debug_shared_passes(out): the passes over tables that shared scans of
+ * this process have enqueued so far: out[0] by table lookup, out[1]
+ * interpreted. */
+esc_status esc_debug_shared_passes(uint64_t *out);
 /* esc_debug_mlp_give_up(wait): in the checked build, the wait of this number
  * (from 1) of every block of the following MLP kernels gives up, as if its
  * limit had passed; 0 turns it off.  ESC_EINVAL in the release build. */

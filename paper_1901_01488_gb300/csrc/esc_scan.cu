@@ -2550,11 +2550,15 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
 // predicates 614-825 / 593-976, 8 802-815 / 819-1173, 10 610-816 / 1229-1506;
 // 8M: 8 145-148 / 129-177, 10 119-148 / 185-222, 12 143-147 / 235-256, 16
 // 122-152 / 285-301; 1M: 10 51-56 / 44-51, 12 56 / 52-55, 16 52-60 / 62-64, 32
-// 67-70 / 102-110; 100K: 16 41-47 / 36-38, 32 51 / 55-61.
-inline bool lookup_pays(int32_t n, uint64_t rows) {
-  const uint64_t work = rows * (uint64_t)n;
-  return n >= 32 || (n >= 12 && work >= 16000000u) || (n >= 8 && work >= 80000000u);
+// 67-70 / 102-110; 100K: 16 41-47 / 36-38, 32 49 / 59; 10K: 32 49 / 50, 64 56 /
+// 78; 1K: 32 50 / 40, 64 56 / 54 (the call alone 99 / 81), 128 74 / 83.
+inline bool lookup_pays(size_t n, uint64_t rows) {
+  const uint64_t work = rows * n;
+  return n >= 128 || (n >= 32 && rows >= 10000u) || (n >= 12 && work >= 16000000u) || (n >= 8 && work >= 80000000u);
 }
+
+// Shared passes enqueued by this process: by lookup, interpreted (esc_debug_shared_passes).
+static std::atomic<uint64_t> g_shared_passes[2];
 
 // One shared scan: `n` count-only predicates of table t whose read columns
 // (union `ucols`, table column indices) fit one stage layout.  Predicates that
@@ -2582,14 +2586,19 @@ static esc_status run_shared_group(const esc_table *t, const esc_pred *const *pr
   if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_selectivity_shared_async: ") + cudaGetErrorString(e));
 
   std::vector<int32_t> rest;   // predicates left to the interpreter
-  if (t->nrows > 0 && lookup_pays(n, t->nrows)) {
+  if (t->nrows > 0 && lookup_pays((size_t)n, t->nrows)) {
     std::unique_ptr<BoxPlan, void (*)(BoxPlan *)> plan(new_box_plan(), free_box_plan);
     std::vector<int32_t> in;   // the plan's predicates
     auto flush = [&]() -> esc_status {
+      // (the rule again for what decomposed, or the last pass left: a few
+      // predicates are better added to the interpreter's pass than given one.
+      // 32 predicates on 100K rows of which 10 decompose: 132 us for two
+      // passes, 111 for one)
       bool done = in.empty();
-      if (!done) {
+      if (!done && lookup_pays(in.size(), t->nrows)) {
         const esc_status fs = run_boxes(plan.get(), t, d->sms, counts, hdr, st, &done);
         if (fs != ESC_OK) return fs;
+        if (done) g_shared_passes[0].fetch_add(1, std::memory_order_relaxed);
       }
       if (!done) rest.insert(rest.end(), in.begin(), in.end());
       in.clear();
@@ -2647,6 +2656,7 @@ static esc_status run_shared_group(const esc_table *t, const esc_pred *const *pr
       const uint32_t grid = std::min<uint32_t>((uint32_t)(d->sms * d->blocks_per_sm), Y.nunits);
       shared_kernel<<<grid, kThreads, SharedSmem::total, st>>>(L);
       e = cudaGetLastError();
+      g_shared_passes[1].fetch_add(1, std::memory_order_relaxed);
     }
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(dev_counts, counts, (size_t)n * 8, cudaMemcpyDeviceToDevice, st);
@@ -2661,6 +2671,13 @@ static esc_status run_shared_group(const esc_table *t, const esc_pred *const *pr
   }
 #endif
   if (e != cudaSuccess) return fail(ESC_ECUDA, std::string("esc_selectivity_shared_async: ") + cudaGetErrorString(e));
+  return ESC_OK;
+}
+
+esc_status esc_debug_shared_passes(uint64_t *out) {
+  if (!out) return fail(ESC_EINVAL, "esc_debug_shared_passes: out is NULL");
+  for (int k = 0; k < 2; ++k) out[k] = g_shared_passes[k].load(std::memory_order_relaxed);
+  clear_error();
   return ESC_OK;
 }
 

@@ -91,6 +91,7 @@ _sig = {
     "esc_debug_mlp_give_up": ([ctypes.c_uint32], _S),
     "esc_debug_shrink_table": ([ctypes.c_uint32], _S),
     "esc_debug_fail_host_allocs": ([ctypes.c_int32], _S),
+    "esc_debug_shared_passes": ([ctypes.POINTER(ctypes.c_uint64)], _S),
     "esc_debug_write_units": ([ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32)], _S),
     "esc_build_checked": ([ctypes.POINTER(ctypes.c_int32)], _S),
     "esc_mlp_forward": ([_P, ctypes.c_uint64, _P, _P, _P, _P], _S),
@@ -411,6 +412,13 @@ def esc_debug_shrink_table(chunks: int) -> None:
 
 def esc_debug_fail_host_allocs(n: int) -> None:
     _check(_lib.esc_debug_fail_host_allocs(n), "esc_debug_fail_host_allocs")
+
+
+def esc_debug_shared_passes() -> Tuple[int, int]:
+    """Shared passes enqueued so far: (by table lookup, interpreted)."""
+    out = (ctypes.c_uint64 * 2)()
+    _check(_lib.esc_debug_shared_passes(out), "esc_debug_shared_passes")
+    return out[0], out[1]
 
 
 def esc_debug_write_units(nrows: int, slots: int) -> Tuple[int, int, int]:

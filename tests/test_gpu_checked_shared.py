@@ -20,7 +20,8 @@ def run(args, timeout=900):
     return r.stdout
 
 
-@pytest.mark.parametrize("module", ["test_gpu_shared_boxes.py", "test_gpu_shared_buckets.py"])
+@pytest.mark.parametrize("module", ["test_gpu_shared_boxes.py", "test_gpu_shared_buckets.py",
+                                    "test_gpu_shared_rule.py"])
 def test_every_path(module):
     """Rows' words in registers or shared by lanes, with and without buckets, ragged tables, cuts sorted on the
     GPU, passes at their limits, predicates left to the interpreter."""
@@ -35,7 +36,7 @@ import torch
 from paper_1901_01488_gb300 import esc
 
 assert esc.esc_build_checked()
-rows = 5000
+rows = 12000
 a = (torch.arange(rows, dtype=torch.int32, device="cuda") * 7919) % 3000
 t = esc.Table([("a", "i32", a)], rows)
 for n in (40, 700):          # rows' words in registers; shared by lanes
