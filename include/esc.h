@@ -272,6 +272,13 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
 esc_status esc_selectivity_shared_async(const esc_table *table, const esc_pred *const *preds, int32_t n,
                                         uint64_t *dev_counts, void *stream);
 
+/* The device memory, in bytes, that a shared scan of n predicates takes from
+ * the library's stream-ordered pool at most while it runs, whatever the
+ * predicates (its passes follow one another): the programs, and for passes
+ * by table lookup the tests, their bounds and a table of at most 64 MB.  For
+ * callers that admit work by memory.  ESC_EINVAL for n < 1. */
+esc_status esc_shared_scratch_bytes(int32_t n, uint64_t *bytes);
+
 /* One-shot form of the above: prepares, runs, synchronises and destroys.
  * counts is a host array of n entries. */
 esc_status esc_selectivity_batch(const esc_table *const *tables, const esc_pred *const *preds,

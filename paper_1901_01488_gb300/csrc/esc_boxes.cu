@@ -999,6 +999,22 @@ void make_buckets(Operand &o, const std::vector<int64_t> &cuts, uint32_t most, s
 
 }  // namespace
 
+// (the blocks that run_boxes places, each for the most it can hold)
+uint64_t box_scratch_bound(uint64_t n) {
+  constexpr uint64_t kPredCuts = 2 * kMaxPool + 2 * kMaxInstr;   // a list's value makes two cuts, a range's bounds one each
+  constexpr uint64_t kOthers = (uint64_t)kMaxOperands * 257;     // u8 operands; the interval below each one's cuts
+  const uint64_t boxes = std::min<uint64_t>(n * kMaxBoxes, kMaxPassBoxes), words = (boxes + 31) / 32;
+  // p predicates with cuts have as many boxes at least, and the more boxes the
+  // fewer intervals fit the largest table
+  uint64_t intervals = 0;
+  for (uint64_t p = 0; p <= n; ++p)
+    intervals = std::max(intervals, std::min(kOthers + kPredCuts * p, kMaxTableBytes / (4 * ((p + 31) / 32 + 3))));
+  const uint64_t table = std::min(kMaxTableBytes, intervals * (words + 3) * 4);
+  const uint64_t tests = n * kMaxInstr * sizeof(BoxTest), refs = n * kMaxBoxes * kMaxInstr * 4, pool = n * kMaxPool * 8;
+  const uint64_t cuts = intervals * (8 + 16);   // unsorted; sorted and padded (to less than twice 8 bytes or 4 times 4)
+  return table + tests + refs + pool + boxes * 13 + cuts + kBucketBytes + kMaxOperands * (sizeof(SortJob) + 32) + 16 * 256;
+}
+
 esc_status run_boxes(BoxPlan *P, const esc_table *t, int sms, unsigned long long *counts, ScratchHdr *hdr,
                      cudaStream_t st, bool *done) {
   *done = false;

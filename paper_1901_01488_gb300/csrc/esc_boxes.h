@@ -38,6 +38,9 @@ BoxFit add_predicate(BoxPlan *plan, const esc_pred *p, uint32_t index);
 esc_status run_boxes(BoxPlan *plan, const esc_table *t, int sms, unsigned long long *counts, ScratchHdr *hdr,
                      cudaStream_t st, bool *done);
 
+// Device memory that a pass over at most n predicates allocates, at most.
+uint64_t box_scratch_bound(uint64_t n);
+
 // Stream-ordered allocation from the library's device pool (esc_scan.cu).
 esc_status alloc_async(void **p, size_t bytes, cudaStream_t st);
 

@@ -2674,6 +2674,14 @@ static esc_status run_shared_group(const esc_table *t, const esc_pred *const *pr
   return ESC_OK;
 }
 
+esc_status esc_shared_scratch_bytes(int32_t n, uint64_t *bytes) {
+  if (n < 1 || !bytes) return fail(ESC_EINVAL, "esc_shared_scratch_bytes: need n >= 1 and bytes");
+  const uint64_t k = std::min<uint64_t>((uint64_t)n, kSharedMaxQueries);   // passes follow one another
+  *bytes = 1024 + k * (sizeof(Query) + 8) + box_scratch_bound(k);
+  clear_error();
+  return ESC_OK;
+}
+
 esc_status esc_debug_shared_passes(uint64_t *out) {
   if (!out) return fail(ESC_EINVAL, "esc_debug_shared_passes: out is NULL");
   for (int k = 0; k < 2; ++k) out[k] = g_shared_passes[k].load(std::memory_order_relaxed);

@@ -92,6 +92,7 @@ _sig = {
     "esc_debug_shrink_table": ([ctypes.c_uint32], _S),
     "esc_debug_fail_host_allocs": ([ctypes.c_int32], _S),
     "esc_debug_shared_passes": ([ctypes.POINTER(ctypes.c_uint64)], _S),
+    "esc_shared_scratch_bytes": ([ctypes.c_int32, ctypes.POINTER(ctypes.c_uint64)], _S),
     "esc_debug_write_units": ([ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32)], _S),
     "esc_build_checked": ([ctypes.POINTER(ctypes.c_int32)], _S),
     "esc_mlp_forward": ([_P, ctypes.c_uint64, _P, _P, _P, _P], _S),
@@ -331,6 +332,13 @@ def esc_selectivity_shared_async(table: int, preds: Sequence[int], dev_counts: t
     pa = (_P * n)(*preds)
     _check(_lib.esc_selectivity_shared_async(table, pa, n, dev_counts.data_ptr(), _stream(stream)),
            "esc_selectivity_shared_async")
+
+
+def esc_shared_scratch_bytes(n: int) -> int:
+    """Device memory a shared scan of n predicates takes at most while it runs."""
+    out = ctypes.c_uint64(0)
+    _check(_lib.esc_shared_scratch_bytes(n, ctypes.byref(out)), "esc_shared_scratch_bytes")
+    return out.value
 
 
 def esc_bitmap_build(dim: int, pred: int, dev_bitmap: torch.Tensor, stream=None) -> int:

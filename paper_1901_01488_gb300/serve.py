@@ -5,11 +5,11 @@ a selection, Sec. 2); this is the serving pattern around it.  Requests
 (table, predicate) arrive over time.  A host loop keeps `streams` waves in
 flight: whenever a stream is free it admits every request that has arrived,
 up to `max_batch`, within the device-memory budget (each request reserves the scratch and output bytes
-its materialisation needs) and within `max_wave_rows` table rows scanned (a
+its materialisation needs, and a wave what its shared passes need) and within `max_wave_rows` table rows scanned (a
 wave's requests complete together, so one long wave would hold back every
 short request in it), and launches them: count requests on one table, when
-at least `shared_min` of them arrived together, share one pass over it
-(esc_selectivity_shared_async); the others run as one batch
+at least `shared_min` of them arrived together and the pass's scratch fits the
+budget, share one pass over it (esc_selectivity_shared_async); the others run as one batch
 (esc_selectivity_batch_async), or as a plain call when only one is left.
 Waves on different streams overlap on the GPU.  A request's predicate is
 compiled when it arrives, on the polling thread by default (about 8 us);
@@ -126,6 +126,25 @@ def wave_groups(batch: Sequence[Request], shared_min: int) -> Tuple[List[List[Re
     return groups, [r for r in batch if id(r) not in shared]
 
 
+def fit_groups(groups: List[List[Request]], rest: List[Request], room: int,
+               scratch: Callable[[int], int]) -> Tuple[List[List[Request]], List[Request], int]:
+    """Keeps the shared passes whose scratch (`scratch` of their number of
+    requests) fits in `room` bytes; the others' requests join the batch, in
+    arrival order.  A wave's passes follow one another on its stream, so it
+    holds the largest one's scratch at a time, returned as the third value."""
+    kept, extra, moved = [], 0, []
+    for g in groups:
+        need = scratch(len(g))
+        if need <= room:
+            kept.append(g)
+            extra = max(extra, need)
+        else:
+            moved.extend(g)
+    if moved:
+        rest = sorted(rest + moved, key=lambda r: r.arrival)
+    return kept, rest, extra
+
+
 class Server:
     def __init__(self, esc, tables, mem_budget: int = 8 << 30, max_batch: int = 512, streams: int = 2,
                  device="cuda", shared_min: int = 8, compile_threads: int = 0,
@@ -211,6 +230,9 @@ class Server:
         esc = self.esc
         # shared passes first (one per table), then the rest as one batch
         groups, rest_reqs = wave_groups(batch, self.shared_min)
+        groups, rest_reqs, extra = fit_groups(groups, rest_reqs, self.budget - self.in_flight_bytes - nbytes,
+                                              esc.esc_shared_scratch_bytes)
+        nbytes += extra
         batch = [r for g in groups for r in g] + rest_reqs
         nshared = len(batch) - len(rest_reqs)
         preds = []
