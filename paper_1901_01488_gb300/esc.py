@@ -121,12 +121,19 @@ def _check(status: int, where: str, ok=(ESC_OK,)) -> int:
     return status
 
 
+# The current stream's handle without the Stream object around it; not part of
+# PyTorch's public interface, so that it may be missing.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
         if not torch.cuda.is_initialized():
             torch.cuda.init()
-        # the current stream's handle, without the Stream object around it
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if _raw_stream is None or _get_device is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_get_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
