@@ -59,7 +59,8 @@ constexpr uint32_t kBlock = 128 * 128;       // bytes of a 128-row operand block
 // before it adds anything that depends on the wait, waits once more for those
 // in flight, and leaves NaN in the outputs it did not compute (y) or in
 // loss_sum.  (Agreeing on it costs nothing that shows in the gradient, 28.7 us
-// a step of 4096 samples; predicting 1M samples takes 147.4 us instead of 147.2.)
+// a step of 4096 samples; predicting 1M samples takes 147.4 us instead of 147.2,
+// and 147.9 with the search for infinite weights below.)
 __device__ ScratchHdr g_mlp_hdr;
 #ifdef ESC_CHECKED
 __device__ uint32_t g_mlp_give_up;   // test hook: each block's wait of this number gives up (0: none)
@@ -186,20 +187,50 @@ struct MlpVectors {
   float pad[3];
 };
 
-// W1 (one block) and W2 (two) to shared memory, and the float32 vectors.
+// W1 (one block) and W2 (two) to shared memory, and the float32 vectors.  True
+// when this thread has met an infinity in W2: the tensor cores would multiply
+// it with z1's three parts, of which some are 0 (0 times it is NaN, and the
+// unit would count as inactive), so that such weights take plain arithmetic.
+// (A negative infinity makes its unit inactive either way.)
 template <int NT>
-__device__ __forceinline__ void load_weights(uint8_t *w1, uint8_t *w2, MlpVectors &V, const uint16_t *wbf, const float *pf) {
+__device__ __forceinline__ bool load_weights(uint8_t *w1, uint8_t *w2, MlpVectors &V, const uint16_t *wbf, const float *pf) {
   const bool vec = ((uintptr_t)wbf & 15u) == 0;
   for (uint32_t i = threadIdx.x; i < kH * kIn / 8; i += NT)
     *reinterpret_cast<uint4 *>(chunk(w1, i >> 3, i & 7u)) = load8(wbf + kW1 + 8 * i, vec);
-  for (uint32_t i = threadIdx.x; i < kH * kH / 8; i += NT)
-    *reinterpret_cast<uint4 *>(chunk(w2 + ((i >> 3) & 1u) * kBlock, i >> 4, i & 7u)) = load8(wbf + kW2 + 8 * i, vec);
+  bool inf = false;
+  for (uint32_t i = threadIdx.x; i < kH * kH / 8; i += NT) {
+    const uint4 w = load8(wbf + kW2 + 8 * i, vec);
+    *reinterpret_cast<uint4 *>(chunk(w2 + ((i >> 3) & 1u) * kBlock, i >> 4, i & 7u)) = w;
+    const uint32_t most = __vmaxs2(__vmaxs2(w.x, w.y), __vmaxs2(w.z, w.w));   // (positive NaN, above infinity: no matter)
+    inf = inf || (most & 0xffffu) - 0x7f80u < 0x80u || (most >> 16) - 0x7f80u < 0x80u;
+  }
   for (uint32_t i = threadIdx.x; i < kH; i += NT) {
     V.b1[i] = pf[kB1 + i];
     V.b2[i] = pf[kB2 + i];
     V.w3[i] = bf(wbf[kW3 + i]);
   }
   if (threadIdx.x == 0) V.b3 = pf[kB3];
+  return inf;
+}
+
+// Value i of a row of an operand block (two blocks for 128 columns).
+__device__ __forceinline__ float operand(const uint8_t *blocks, uint32_t row, uint32_t i) {
+  const uint8_t *b = blocks + (i >> 6) * kBlock + row * 128u + ((((i >> 3) & 7u) ^ (row & 7u)) << 4) + 2u * (i & 7u);
+  return bf(*reinterpret_cast<const uint16_t *>(b));
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  return v;
+}
+// relu of one unit of a layer by plain arithmetic: its row of weights times n values, and its bias.
+template <typename V>
+__device__ __forceinline__ float plain_unit(const uint8_t *w, uint32_t unit, float bias, uint32_t n, V value) {
+  float a = bias;
+#pragma unroll 1
+  for (uint32_t k = 0; k < n; ++k) a = fmaf(operand(w, unit, k), value(k), a);
+  return fmaxf(a, 0.0f);
 }
 
 // This thread's chunks of a tile's features (samples past the batch: 0).
@@ -330,7 +361,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  load_weights<kFwdThreads>(sm + FwdSmem::w1, sm + FwdSmem::w2, V, wbf, pf);
+  const bool inf = load_weights<kFwdThreads>(sm + FwdSmem::w1, sm + FwdSmem::w2, V, wbf, pf);
   store_x<kFwdThreads>(sm + FwdSmem::x, xr);
   fence_proxy_async_smem();
   tc_before_sync();
@@ -409,7 +440,25 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
     for (; s0 < B; s0 += (uint64_t)gridDim.x * kTileS)
       if (half == 0 && s0 + row < B) y[s0 + row] = __int_as_float(0x7fffffff);
   }
-  __syncthreads();
+  // An infinity in W2: once more, sample by sample, thread = unit.  (At the end,
+  // as leaving before the loop cost it registers: 160 us instead of 147.)
+  if (__syncthreads_or(inf)) {
+    float *z1 = ypart, *red = reinterpret_cast<float *>(Z);
+#pragma unroll 1
+    for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS)
+#pragma unroll 1
+      for (uint64_t s = s0; s < B && s < s0 + kTileS; ++s) {
+        if (half == 0) z1[row] = plain_unit(sm + FwdSmem::w1, row, V.b1[row], kIn, [&](uint32_t m) { return bf(x[s * kIn + m]); });
+        __syncthreads();
+        if (half == 0) {
+          const float v = warp_sum(V.w3[row] * plain_unit(sm + FwdSmem::w2, row, V.b2[row], kH, [&](uint32_t k) { return z1[k]; }));
+          if ((threadIdx.x & 31u) == 0) red[warp] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) y[s] = (red[0] + red[1]) + (red[2] + red[3]) + V.b3;
+      }
+    __syncthreads();
+  }
   if (warp == 0) tmem_free(tm, kFwdCols);
 }
 
@@ -448,33 +497,39 @@ __device__ __forceinline__ void add4(float *p, float a, float b, float c, float 
   }
 }
 
-// Value i of a row of an operand block (two blocks for 128 columns).
-__device__ __forceinline__ float operand(const uint8_t *blocks, uint32_t row, uint32_t i) {
-  const uint8_t *b = blocks + (i >> 6) * kBlock + row * 128u + ((((i >> 3) & 7u) ^ (row & 7u)) << 4) + 2u * (i & 7u);
-  return bf(*reinterpret_cast<const uint16_t *>(b));
-}
-
 // Adds one sample's gradient (the tile's row r) by plain arithmetic, unit by
 // unit: for samples with an infinity or NaN among the products' factors.  Those
 // are left out of the products, where 0 times such a factor would reach every
-// unit, active or not.  `s`: 384 floats of scratch in shared memory; the whole
-// block calls.
-__device__ __noinline__ void add_sample(const uint8_t *sm, const MlpVectors &V, float *s, uint32_t r, float dy, float *grad) {
+// unit, active or not.  `dy`: 2 / B times its residual; with `target` (an
+// infinity in W2, see load_weights) the residual is found here, dy is 2 / B,
+// and b3's gradient and the loss are added as well.  `s`: 384 floats of scratch
+// in shared memory; the whole block calls.
+__device__ __noinline__ void add_sample(const uint8_t *sm, const MlpVectors &V, float *s, uint32_t r, float dy,
+                                        const float *target, float *grad, float *loss_sum) {
   const uint8_t *w1 = sm + GradSmem::w1, *w2 = sm + GradSmem::w2, *x = sm + GradSmem::x;
   float *z1 = s, *d2 = s + kH, *d1 = s + 2 * kH;
   const uint32_t j = threadIdx.x & 127u, quarter = threadIdx.x >> 7;
-  if (quarter == 0) {
-    float a = V.b1[j];
-    for (uint32_t m = 0; m < kIn; ++m) a = fmaf(operand(w1, j, m), operand(x, r, m), a);
-    z1[j] = fmaxf(a, 0.0f);
-  }
+  if (quarter == 0) z1[j] = plain_unit(w1, j, V.b1[j], kIn, [&](uint32_t m) { return operand(x, r, m); });
   __syncthreads();
+  float z2 = 0.0f;
+  if (quarter == 0) z2 = plain_unit(w2, j, V.b2[j], kH, [&](uint32_t k) { return z1[k]; });
+  if (target) {
+    if (quarter == 0) {
+      const float v = warp_sum(V.w3[j] * z2);
+      if ((j & 31u) == 0) d1[j >> 5] = v;
+    }
+    __syncthreads();
+    const float e = (d1[0] + d1[1]) + (d1[2] + d1[3]) + V.b3 - *target;
+    dy *= e;
+    if (threadIdx.x == 0) {
+      atomicAdd(&grad[kB3], dy);
+      atomicAdd(loss_sum, e * e);
+    }
+  }
   if (quarter == 0) {
-    float a = V.b2[j];
-    for (uint32_t k = 0; k < kH; ++k) a = fmaf(operand(w2, j, k), z1[k], a);
-    d2[j] = a > 0.0f ? dy * V.w3[j] : 0.0f;
+    d2[j] = z2 > 0.0f ? dy * V.w3[j] : 0.0f;
     atomicAdd(&grad[kB2 + j], d2[j]);
-    atomicAdd(&grad[kW3 + j], dy * fmaxf(a, 0.0f));
+    atomicAdd(&grad[kW3 + j], dy * z2);
   }
   __syncthreads();
   for (uint32_t k = 32 * quarter; k < 32 * quarter + 32; ++k) atomicAdd(&grad[kW2 + j * kH + k], d2[j] * z1[k]);
@@ -511,7 +566,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     bad[0] = bad[1] = bad[2] = bad[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  load_weights<kGradThreads>(sm + GradSmem::w1, sm + GradSmem::w2, V, wbf, pf);
+  const bool inf = load_weights<kGradThreads>(sm + GradSmem::w1, sm + GradSmem::w2, V, wbf, pf);
 #pragma unroll
   for (uint32_t c = 0; c < 2; ++c) *reinterpret_cast<uint4 *>(chunk(E, row, 2 * quarter + c)) = make_uint4(0, 0, 0, 0);
   store_x<kGradThreads>(sm + GradSmem::x, xr);
@@ -545,7 +600,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     store_split32<true>(R, quarter, row, z1);
     fence_proxy_async_smem();
     tc_before_sync();
-    ok = __syncthreads_and(ok) != 0;
+    ok = __syncthreads_and(ok && !inf) != 0;
     if (!ok) break;
     if (threadIdx.x == 0) {
       tc_after_sync();
@@ -665,7 +720,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       tc_commit(&bar[0]);
     }
     // meanwhile gW2 goes out: row j is this thread's lane
-    const float w3 = V.w3[row];
+    const float w3 = fabsf(V.w3[row]) <= FLT_MAX ? V.w3[row] : 0.0f;   // (otherwise every sample was left out)
     float2 dot = make_float2(0.0f, 0.0f);
     load_sum32(mine, v);
     {
@@ -721,7 +776,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     if (left.x | left.y | left.z | left.w) {
       __syncthreads();   // (part has been read)
       for (uint32_t r = 0; r < kTileS; ++r)
-        if ((bad[r >> 5] >> (r & 31u)) & 1u) add_sample(sm, V, part, r, bad_dy[r], grad);
+        if ((bad[r >> 5] >> (r & 31u)) & 1u) add_sample(sm, V, part, r, bad_dy[r], nullptr, grad, loss_sum);
       if (threadIdx.x < 4) bad[threadIdx.x] = 0;
     }
     store_x<kGradThreads>(sm + GradSmem::x, xr);
@@ -733,7 +788,18 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   if (!ok) {
     mbar_wait(&bar[0], ph0 ^ 1u, &g_mlp_hdr);   // the products in flight
     mbar_wait(&bar[1], ph1 ^ 1u, &g_mlp_hdr);
-    lsum = __int_as_float(0x7fffffff);
+    if (__syncthreads_or(inf)) {   // an infinity in W2 (the first tile has ended here): sample by sample
+#pragma unroll 1
+      for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
+#pragma unroll 1
+        for (uint32_t r = 0; r < kTileS && s0 + r < B; ++r) add_sample(sm, V, part, r, 2.0f / (float)B, t + s0 + r, grad, loss_sum);
+        load_x<kGradThreads>(x, B, s0 + (uint64_t)gridDim.x * kTileS, vec, xr);
+        store_x<kGradThreads>(sm + GradSmem::x, xr);
+        __syncthreads();
+      }
+    } else {
+      lsum = __int_as_float(0x7fffffff);
+    }
   }
   if (quarter == 0) {
 #pragma unroll

@@ -109,3 +109,74 @@ def test_dead_unit_with_a_bad_bias():
     assert torch.equal(out[0][:-1], out[1][:-1])
     assert abs(out[0][-1] - out[1][-1]).item() <= 2.0 ** -21 * (2 / B * (layers(P, x)[6] + np.abs(t))).sum()
     assert out[1][b2 + 3].item() == 0.0 and out[1][b2 + 128 + 3].item() == 0.0
+
+
+def expected(x, t, p):
+    """y and the gradient with infinite parameters, in float64: 0 times infinity is NaN, which ReLU takes to 0."""
+    P = {k: v.double() for k, v in omlp_torch(p).items()}
+    x = x.double()
+    relu = lambda a: torch.where(a > 0, a, torch.zeros((), dtype=torch.float64))
+    prod = lambda a, w: (a[:, None, :] * w[None, :, :]).sum(2)        # (a library's product may skip zeros)
+    a1 = prod(x, P["W1"]) + P["b1"]
+    z1 = relu(a1)
+    a2 = prod(z1, P["W2"]) + P["b2"]
+    z2 = relu(a2)
+    y = (z2 * P["w3"]).sum(1) + P["b3"]
+    dy = 2.0 / len(t) * (y - t.double())
+    d2 = torch.where(a2 > 0, dy[:, None] * P["w3"], torch.zeros((), dtype=torch.float64))
+    d1 = torch.where(a1 > 0, prod(d2, P["W2"].T.contiguous()), torch.zeros((), dtype=torch.float64))
+    g = {"W1": prod(d1.T, x.T.contiguous()), "b1": d1.sum(0), "W2": prod(d2.T, z1.T.contiguous()), "b2": d2.sum(0),
+         "w3": prod(dy[None], z2.T.contiguous())[0], "b3": dy.sum()[None]}
+    return y, g
+
+
+def omlp_torch(p):
+    out, o = {}, 0
+    for name, s in omlp.sizes().items():
+        n = int(np.prod(s))
+        out[name] = p[o:o + n].reshape(s)
+        o += n
+    return out
+
+
+@pytest.mark.parametrize("where", ["W2", "W2 unreached", "-W2", "w3", "w3 dead"])
+@pytest.mark.parametrize("B", [1, 130])
+def test_infinite_weights(B, where):
+    """Small whole numbers throughout, so that the parts of an activation that are 0 (all but the
+    first) and every sum are exact: finite values are compared exactly."""
+    from paper_1901_01488_gb300 import esc
+    rng = np.random.default_rng(B)
+    p = torch.from_numpy(rng.integers(-2, 3, esc.MLP_PARAMS).astype(np.float32))
+    P = omlp_torch(p)
+    P["b1"][5], P["W1"][5] = 3.0, 0.0               # an active unit of the first layer, and an inactive one
+    P["b1"][6], P["W1"][6] = -3.0, 0.0
+    P["b2"][9], P["W2"][9] = -8.0, 0.0              # a unit that no sample activates
+    inf = float("inf")
+    if where == "W2":
+        P["W2"][7][5] = inf
+        P["w3"][7] = 2.0
+    elif where == "W2 unreached":
+        P["W2"][7][6] = inf                          # 0 times it: NaN, so the unit is inactive
+    elif where == "-W2":
+        P["W2"][7][5] = -inf
+    elif where == "w3":
+        P["w3"][7] = inf
+    else:
+        P["w3"][9] = inf
+    x = torch.from_numpy(rng.integers(0, 2, (B, 64)).astype(np.float32))
+    t = torch.from_numpy(rng.integers(-3, 4, B).astype(np.float32))
+    y, g = expected(x, t, p)
+    dx, dw, dp = x.to(torch.bfloat16).view(torch.int16).cuda(), p.to(torch.bfloat16).view(torch.int16).cuda(), p.cuda()
+    out = torch.full((B,), 7.0, device="cuda")
+    esc.esc_mlp_forward(dx, dw, dp, out)
+    same = lambda a, b: torch.equal(torch.isfinite(a), torch.isfinite(b))
+    out = out.cpu().double()
+    assert same(out, y) and torch.equal(out[torch.isfinite(y)], y[torch.isfinite(y)])
+    assert torch.equal(out == inf, y == inf) and torch.equal(out == -inf, y == -inf)
+    grad, loss = torch.zeros(esc.MLP_PARAMS, device="cuda"), torch.zeros(1, device="cuda")
+    esc.esc_mlp_grad(dx, dt := t.cuda(), dw, dp, grad, loss)
+    got = omlp_torch(grad.cpu().double())
+    for k, want in g.items():
+        assert same(got[k], want), k
+        f = torch.isfinite(want)
+        assert bool(((got[k] - want).abs()[f] <= 2.0 ** -14 * (want.abs()[f] + 1e4)).all()), k
