@@ -255,7 +255,8 @@ esc_status esc_batch_destroy(esc_batch *batch);
  * counts to dev_counts and, when dev_done_ns is not NULL, each sub-query's
  * completion time (%globaltimer).  Does not synchronise; `rows` entries with
  * capacity 0 and row_ids NULL are count-only; truncation is not reported
- * (written = min(count, capacity)).  Host arrays may be freed on return. */
+ * (written = min(count, capacity)), nor are device-side timeouts.  Host arrays
+ * may be freed on return. */
 esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc_pred *const *preds,
                                        int32_t n, const esc_rows *rows, uint64_t *dev_counts,
                                        uint64_t *dev_done_ns, void *stream);
@@ -268,6 +269,7 @@ esc_status esc_selectivity_batch_async(const esc_table *const *tables, const esc
  * order of preds, when the stream reaches that point.  Predicates are taken
  * in passes whose read columns fit the 16 stage slots, at most 2048 per
  * pass.  Does not synchronise; host arrays may be freed on return.
+ * Device-side timeouts are not reported by this call.
  * ESC_EINVAL for a NULL argument or a predicate of another table. */
 esc_status esc_selectivity_shared_async(const esc_table *table, const esc_pred *const *preds, int32_t n,
                                         uint64_t *dev_counts, void *stream);

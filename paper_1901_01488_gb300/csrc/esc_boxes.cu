@@ -508,11 +508,11 @@ struct TileRing {
     return mbar_wait(&full[j % kBoxStages], (j / kBoxStages) & 1u, L.hdr);
   }
   // Barrier after the stage's last use; then the copy of tile j + kBoxStages
-  // goes into it.  False (for the whole block) when a warp gave up waiting:
-  // the other copies in flight are waited for, bounded, and the block leaves.
+  // goes into it.  False (for the whole block) when a warp gave up waiting: the
+  // copies in flight, this tile's too, are waited for, bounded, and the block leaves.
   __device__ __forceinline__ bool release(const BoxLaunch &L, uint32_t j, bool ok) const {
     if (!__syncthreads_and(ok)) {
-      for (uint32_t k = j + 1; k < total && k < j + kBoxStages; ++k) wait(L, k);
+      for (uint32_t k = j; k < total && k < j + kBoxStages; ++k) wait(L, k);
       return false;
     }
     if (threadIdx.x < 32 && j + kBoxStages < total) issue(L, j + kBoxStages);
