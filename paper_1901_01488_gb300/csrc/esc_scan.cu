@@ -540,8 +540,8 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1) scan_kernel(const __grid_con
     block_sum[0] = block_sum[1] = block_sum[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // a single sub-query is staged once, by the consumers, while the producer
-  // starts the first copies
+  // a single sub-query is staged once, by the consumers; the producer, which
+  // reads it from the parameters, starts its copies after the same barrier
   if (single && warp > 0) {
     copy_query(reinterpret_cast<uint8_t *>(qslot), L.q0, threadIdx.x - 32, 32 * NC);
   }
