@@ -58,9 +58,9 @@ constexpr uint32_t kBlock = 128 * 128;       // bytes of a 128-row operand block
 // return): the outputs say so.  The block stops before its next products and
 // before it adds anything that depends on the wait, waits once more for those
 // in flight, and leaves NaN in the outputs it did not compute (y) or in
-// loss_sum.  (Agreeing on it costs nothing that shows in the gradient, 28.7 us
-// a step of 4096 samples; predicting 1M samples takes 147.4 us instead of 147.2,
-// and 147.9 with the search for infinite weights below.)
+// loss_sum.  (With this and the search for infinite weights below, 1M
+// predictions take 146.4 us, 147.5 before; a training step of 4096 samples 29.0
+// us on both sides.)
 __device__ ScratchHdr g_mlp_hdr;
 #ifdef ESC_CHECKED
 __device__ uint32_t g_mlp_give_up;   // test hook: each block's wait of this number gives up (0: none)
@@ -184,7 +184,8 @@ __device__ __forceinline__ uint8_t *chunk(uint8_t *block, uint32_t row, uint32_t
 struct MlpVectors {
   float b1[kH], b2[kH], w3[kH];
   float b3;
-  float pad[3];
+  uint32_t inf;   // forward kernel: an infinity in W2
+  float pad[2];
 };
 
 // W1 (one block) and W2 (two) to shared memory, and the float32 vectors.  True
@@ -197,20 +198,22 @@ __device__ __forceinline__ bool load_weights(uint8_t *w1, uint8_t *w2, MlpVector
   const bool vec = ((uintptr_t)wbf & 15u) == 0;
   for (uint32_t i = threadIdx.x; i < kH * kIn / 8; i += NT)
     *reinterpret_cast<uint4 *>(chunk(w1, i >> 3, i & 7u)) = load8(wbf + kW1 + 8 * i, vec);
-  bool inf = false;
+  uint32_t most = 0;   // the largest of either half's values (as signed numbers: infinity, or a NaN, which is no matter)
   for (uint32_t i = threadIdx.x; i < kH * kH / 8; i += NT) {
     const uint4 w = load8(wbf + kW2 + 8 * i, vec);
     *reinterpret_cast<uint4 *>(chunk(w2 + ((i >> 3) & 1u) * kBlock, i >> 4, i & 7u)) = w;
-    const uint32_t most = __vmaxs2(__vmaxs2(w.x, w.y), __vmaxs2(w.z, w.w));   // (positive NaN, above infinity: no matter)
-    inf = inf || (most & 0xffffu) - 0x7f80u < 0x80u || (most >> 16) - 0x7f80u < 0x80u;
+    most = __vmaxs2(most, __vmaxs2(__vmaxs2(w.x, w.y), __vmaxs2(w.z, w.w)));
   }
   for (uint32_t i = threadIdx.x; i < kH; i += NT) {
     V.b1[i] = pf[kB1 + i];
     V.b2[i] = pf[kB2 + i];
     V.w3[i] = bf(wbf[kW3 + i]);
   }
-  if (threadIdx.x == 0) V.b3 = pf[kB3];
-  return inf;
+  if (threadIdx.x == 0) {
+    V.b3 = pf[kB3];
+    V.inf = 0;
+  }
+  return (most & 0xffffu) >= 0x7f80u || (most >> 16) >= 0x7f80u;
 }
 
 // Value i of a row of an operand block (two blocks for 128 columns).
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
   fence_proxy_async_smem();
   tc_before_sync();
   __syncthreads();
+  if (inf) V.inf = 1;
   tc_after_sync();
   const uint32_t tm = *slot, lanes = tm + ((warp & 3u) << 21);   // + 32 * (warp % 4) lanes
   const uint64_t dw1 = sdesc(smem_addr(sm + FwdSmem::w1)), dw2 = sdesc(smem_addr(sm + FwdSmem::w2)),
@@ -440,9 +444,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
     for (; s0 < B; s0 += (uint64_t)gridDim.x * kTileS)
       if (half == 0 && s0 + row < B) y[s0 + row] = __int_as_float(0x7fffffff);
   }
-  // An infinity in W2: once more, sample by sample, thread = unit.  (At the end,
-  // as leaving before the loop cost it registers: 160 us instead of 147.)
-  if (__syncthreads_or(inf)) {
+  // An infinity in W2: once more, sample by sample, thread = unit.  (Here, by way
+  // of shared memory, as leaving before the loop cost it registers: 160 us
+  // instead of 147.)
+  __syncthreads();
+  if (V.inf) {
     float *z1 = ypart, *red = reinterpret_cast<float *>(Z);
 #pragma unroll 1
     for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS)
