@@ -21,7 +21,7 @@
 // so that only z1, dy z1 and d1 need the split.  A factor of these sums over
 // samples that is infinite or NaN would reach every unit, active or not (0
 // times it is NaN), so such samples take part in them with zeros and are added
-// by plain arithmetic (add_sample): only what they reach becomes non-finite.
+// by plain arithmetic (add_samples): only what they reach becomes non-finite.
 //
 // Shared-memory operands are rows of 128 bytes with 128-byte swizzle (the
 // 16-byte chunk c of row r at c ^ (r % 8)), 64 columns a block of 16 KB per 128
@@ -231,7 +231,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <typename V>
 __device__ __forceinline__ float plain_unit(const uint8_t *w, uint32_t unit, float bias, uint32_t n, V value) {
   float a = bias;
-#pragma unroll 1
+#pragma unroll 8
   for (uint32_t k = 0; k < n; ++k) a = fmaf(operand(w, unit, k), value(k), a);
   return fmaxf(a, 0.0f);
 }
@@ -482,8 +482,9 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
 // and conversions of one tile, the loading of weights, and the fetching of
 // instructions that each block runs once (20 us here by ncu, 24 with 256
 // threads and twice the code, 43 before the tensor cores).  A training step
-// (two fills, this, Adam): 4096 samples 50.5 -> 28.6 us, 20,000 162 -> 47,
-// 65,536 417 -> 76.
+// (two fills, this, Adam): 4096 samples 50.5 -> 29 us, 20,000 162 -> 48, 65,536
+// 417 -> 79.  Of that, the tests for infinities, NaN and waits that gave up are
+// 0.5 us, 1 to 2 and 2 to 4.
 constexpr uint32_t kTgB = 384, kTm = 448, kTgW1 = 448;
 struct GradSmem {
   static constexpr uint32_t w1 = 0, w2 = kBlock, x = 3 * kBlock, e = 4 * kBlock, mask = 5 * kBlock, r = 7 * kBlock,
@@ -503,50 +504,97 @@ __device__ __forceinline__ void add4(float *p, float a, float b, float c, float 
   }
 }
 
-// Adds one sample's gradient (the tile's row r) by plain arithmetic, unit by
-// unit: for samples with an infinity or NaN among the products' factors.  Those
-// are left out of the products, where 0 times such a factor would reach every
-// unit, active or not.  `dy`: 2 / B times its residual; with `target` (an
-// infinity in W2, see load_weights) the residual is found here, dy is 2 / B,
-// and b3's gradient and the loss are added as well.  `s`: 384 floats of scratch
-// in shared memory; the whole block calls.
-__device__ __noinline__ void add_sample(const uint8_t *sm, const MlpVectors &V, float *s, uint32_t r, float dy,
-                                        const float *target, float *grad, float *loss_sum) {
+// Adds the gradient of the tile's rows in `bad` (128 bits) by plain arithmetic,
+// unit by unit: samples with an infinity or NaN among the products' factors.
+// Those are left out of the products, where 0 times such a factor would reach
+// every unit, active or not.  `dy`: 2 / B times their residuals; with `target`
+// (an infinity in W2, see load_weights) the residuals are found here, scale is
+// 2 / B, and b3's gradient and the loss are added as well.  Four rows at a
+// time, one for each 128 threads; `scratch`: shared memory.  The whole block
+// calls, and meets at a barrier before it leaves.  A gradient of 4096 samples
+// takes 35 us with one bad residual and 240 us with nothing but bad ones (19
+// without; 39 either way before the tensor cores), 1M samples 749 us and 12.5 ms
+// (747; 6.1 ms).
+struct PlainRows {
+  float z1[4][kH], d2[4][kH], d1[4][kH], red[4][4];
+  uint8_t row[kTileS];
+};
+__device__ __noinline__ void add_samples(const uint8_t *sm, const MlpVectors &V, uint8_t *scratch, const uint32_t *bad,
+                                         const float *dy, float scale, const float *target, float *grad, float *loss_sum) {
   const uint8_t *w1 = sm + GradSmem::w1, *w2 = sm + GradSmem::w2, *x = sm + GradSmem::x;
-  float *z1 = s, *d2 = s + kH, *d1 = s + 2 * kH;
-  const uint32_t j = threadIdx.x & 127u, quarter = threadIdx.x >> 7;
-  if (quarter == 0) z1[j] = plain_unit(w1, j, V.b1[j], kIn, [&](uint32_t m) { return operand(x, r, m); });
+  PlainRows &P = *reinterpret_cast<PlainRows *>(scratch);
+  const uint32_t j = threadIdx.x & 127u, q = threadIdx.x >> 7;
+  uint32_t n = 0, before = 0;
+  for (uint32_t k = 0; k < 4; ++k) {
+    n += __popc(bad[k]);
+    before += __popc(k < (j >> 5) ? bad[k] : k == (j >> 5) ? bad[k] & ((1u << (j & 31u)) - 1u) : 0u);
+  }
+  if (q == 0 && ((bad[j >> 5] >> (j & 31u)) & 1u)) P.row[before] = (uint8_t)j;
   __syncthreads();
-  float z2 = 0.0f;
-  if (quarter == 0) z2 = plain_unit(w2, j, V.b2[j], kH, [&](uint32_t k) { return z1[k]; });
-  if (target) {
-    if (quarter == 0) {
+  float g2[32], g1[16], gb1 = 0.0f, gb2 = 0.0f, gw3 = 0.0f;   // row j of W2's and W1's gradients, a quarter of each
+#pragma unroll
+  for (int k = 0; k < 32; ++k) g2[k] = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) g1[k] = 0.0f;
+#pragma unroll 1
+  for (uint32_t i = 0; i < n; i += 4) {
+    const uint32_t rows = min(4u, n - i), r = P.row[i + min(q, rows - 1)];
+    const bool mine = q < rows;
+    if (mine) P.z1[q][j] = plain_unit(w1, j, V.b1[j], kIn, [&](uint32_t m) { return operand(x, r, m); });
+    __syncthreads();
+    float z2 = 0.0f, dyr = 0.0f;
+    if (mine) z2 = plain_unit(w2, j, V.b2[j], kH, [&](uint32_t k) { return P.z1[q][k]; });
+    if (target) {
       const float v = warp_sum(V.w3[j] * z2);
-      if ((j & 31u) == 0) d1[j >> 5] = v;
+      if ((j & 31u) == 0) P.red[q][j >> 5] = v;
+      __syncthreads();
+      if (mine) {
+        const float e = (P.red[q][0] + P.red[q][1]) + (P.red[q][2] + P.red[q][3]) + V.b3 - target[r];
+        dyr = e * scale;
+        if (j == 0) {
+          atomicAdd(&grad[kB3], dyr);
+          atomicAdd(loss_sum, e * e);
+        }
+      }
+    } else if (mine) {
+      dyr = dy[r];
+    }
+    if (mine) {
+      const float d = z2 > 0.0f ? dyr * V.w3[j] : 0.0f;
+      P.d2[q][j] = d;
+      gb2 += d;
+      gw3 = fmaf(dyr, z2, gw3);
     }
     __syncthreads();
-    const float e = (d1[0] + d1[1]) + (d1[2] + d1[3]) + V.b3 - *target;
-    dy *= e;
-    if (threadIdx.x == 0) {
-      atomicAdd(&grad[kB3], dy);
-      atomicAdd(loss_sum, e * e);
+    for (uint32_t p = 0; p < rows; ++p) {
+      const float d = P.d2[p][j];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) g2[k] = fmaf(d, P.z1[p][32 * q + k], g2[k]);
     }
+    if (mine) {
+      float g = 0.0f;
+#pragma unroll 8
+      for (uint32_t k = 0; k < kH; ++k) g = fmaf(operand(w2, k, j), P.d2[q][k], g);
+      g = P.z1[q][j] > 0.0f ? g : 0.0f;
+      P.d1[q][j] = g;
+      gb1 += g;
+    }
+    __syncthreads();
+    for (uint32_t p = 0; p < rows; ++p) {
+      const float d = P.d1[p][j];
+      const uint32_t rp = P.row[i + p];
+#pragma unroll
+      for (int m = 0; m < 16; ++m) g1[m] = fmaf(d, operand(x, rp, 16 * q + m), g1[m]);
+    }
+    __syncthreads();
   }
-  if (quarter == 0) {
-    d2[j] = z2 > 0.0f ? dy * V.w3[j] : 0.0f;
-    atomicAdd(&grad[kB2 + j], d2[j]);
-    atomicAdd(&grad[kW3 + j], dy * z2);
-  }
-  __syncthreads();
-  for (uint32_t k = 32 * quarter; k < 32 * quarter + 32; ++k) atomicAdd(&grad[kW2 + j * kH + k], d2[j] * z1[k]);
-  if (quarter == 0) {
-    float g = 0.0f;
-    for (uint32_t i = 0; i < kH; ++i) g = fmaf(operand(w2, i, j), d2[i], g);
-    d1[j] = z1[j] > 0.0f ? g : 0.0f;
-    atomicAdd(&grad[kB1 + j], d1[j]);
-  }
-  __syncthreads();
-  for (uint32_t m = 16 * quarter; m < 16 * quarter + 16; ++m) atomicAdd(&grad[kW1 + j * kIn + m], d1[j] * operand(x, r, m));
+#pragma unroll
+  for (int k = 0; k < 32; ++k) atomicAdd(&grad[kW2 + j * kH + 32 * q + k], g2[k]);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) atomicAdd(&grad[kW1 + j * kIn + 16 * q + m], g1[m]);
+  atomicAdd(&grad[kB1 + j], gb1);
+  atomicAdd(&grad[kB2 + j], gb2);
+  atomicAdd(&grad[kW3 + j], gw3);
   __syncthreads();
 }
 
@@ -559,7 +607,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [2]
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + GradSmem::tmem);
   uint8_t *R = sm + GradSmem::r, *E = sm + GradSmem::e, *mask = sm + GradSmem::mask;
-  uint32_t *bad = reinterpret_cast<uint32_t *>(sm + GradSmem::bad);   // the tile's samples left to add_sample (bits)
+  uint32_t *bad = reinterpret_cast<uint32_t *>(sm + GradSmem::bad);   // the tile's samples left to add_samples (bits)
   float *bad_dy = reinterpret_cast<float *>(sm + GradSmem::bad_dy);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, quarter = warp >> 2, row = threadIdx.x & 127u;
   const bool vec = ((uintptr_t)x & 15u) == 0, gvec = ((uintptr_t)grad & 15u) == 0;
@@ -682,7 +730,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     if (__syncthreads_or(left_out || !ok)) {
       ok = __syncthreads_and(ok) != 0;
       if (!ok) break;
-      // those samples' operands become 0; add_sample makes up for them below
+      // those samples' operands become 0; add_samples makes up for them below
       if (left_out) atomicOr(&bad[row >> 5], 1u << (row & 31u));
       if (quarter == 0) bad_dy[row] = dy;
       __syncthreads();
@@ -780,9 +828,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     }
     const uint4 left = *reinterpret_cast<const uint4 *>(bad);
     if (left.x | left.y | left.z | left.w) {
-      __syncthreads();   // (part has been read)
-      for (uint32_t r = 0; r < kTileS; ++r)
-        if ((bad[r >> 5] >> (r & 31u)) & 1u) add_sample(sm, V, part, r, bad_dy[r], nullptr, grad, loss_sum);
+      add_samples(sm, V, R, bad, bad_dy, 0.0f, nullptr, grad, loss_sum);
       if (threadIdx.x < 4) bad[threadIdx.x] = 0;
     }
     store_x<kGradThreads>(sm + GradSmem::x, xr);
@@ -797,8 +843,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     if (__syncthreads_or(inf)) {   // an infinity in W2 (the first tile has ended here): sample by sample
 #pragma unroll 1
       for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
-#pragma unroll 1
-        for (uint32_t r = 0; r < kTileS && s0 + r < B; ++r) add_sample(sm, V, part, r, 2.0f / (float)B, t + s0 + r, grad, loss_sum);
+        const uint64_t left = B - s0;   // rows of the tile
+        if (threadIdx.x < 4) bad[threadIdx.x] = left >= 32 * threadIdx.x + 32 ? ~0u : left > 32 * threadIdx.x ? (1u << (left & 31u)) - 1u : 0u;
+        __syncthreads();
+        add_samples(sm, V, R, bad, nullptr, inv_b, t + s0, grad, loss_sum);
         load_x<kGradThreads>(x, B, s0 + (uint64_t)gridDim.x * kTileS, vec, xr);
         store_x<kGradThreads>(sm + GradSmem::x, xr);
         __syncthreads();
