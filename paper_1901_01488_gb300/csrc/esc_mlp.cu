@@ -53,15 +53,13 @@ static_assert(kW2 % 8 == 0, "16-byte chunks of W2");
 
 constexpr uint32_t kBlock = 128 * 128;       // bytes of a 128-row operand block (64 columns)
 
-// A wait on the tensor cores that gives up raises its status here, where nothing
-// reads it (these entry points do not synchronise and have no status to
-// return): the outputs say so.  The block stops before its next products and
-// before it adds anything that depends on the wait, waits once more for those
-// in flight, and leaves NaN in the outputs it did not compute (y) or in
-// loss_sum.  (With this and the search for infinite weights below, 1M
-// predictions take 146.4 us, 147.5 before; a training step of 4096 samples 29.0
-// us on both sides.)
-__device__ ScratchHdr g_mlp_hdr;
+// A wait on the tensor cores that gives up raises its status in a header of the
+// block's own, in shared memory (these entry points do not synchronise and have
+// no status to return): the outputs say so.  Later waits of the block then give
+// up at once; it adds and writes nothing that depends on a wait, waits once more
+// for its products in flight, and leaves NaN in the outputs it did not compute
+// (y) or in loss_sum.  (With this and the search for infinite weights below, 1M
+// predictions take 145.8 us, 147.5 before.)
 #ifdef ESC_CHECKED
 __device__ uint32_t g_mlp_give_up;   // test hook: each block's wait of this number gives up (0: none)
 #endif
@@ -89,8 +87,8 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                : "memory");
 }
 // Bounded wait for the phase of parity `parity`; `waits`: this block's so far.
-__device__ __forceinline__ bool tc_wait(uint64_t *bar, uint32_t parity, uint32_t &waits) {
-  const bool done = mbar_wait(bar, parity, &g_mlp_hdr);
+__device__ __forceinline__ bool tc_wait(uint64_t *bar, uint32_t parity, ScratchHdr *hdr, uint32_t &waits) {
+  const bool done = mbar_wait(bar, parity, hdr, kWaitLimitNs, true);
 #ifdef ESC_CHECKED
   if (++waits == *(volatile const uint32_t *)&g_mlp_give_up) return false;   // (the products are done all the same)
 #else
@@ -343,7 +341,8 @@ __device__ __forceinline__ void store_split32(uint8_t *r, uint32_t quarter, uint
 // per SM and four accumulators, 148 us this way.
 struct FwdSmem {
   static constexpr uint32_t w1 = 0, w2 = kBlock, z = 3 * kBlock, x = z, vec = 6 * kBlock, ypart = vec + sizeof(MlpVectors),
-                            bar = ypart + 4 * kTileS, tmem = bar + 8, total = tmem + 8;
+                            bar = ypart + 4 * kTileS, tmem = bar + 8, hdr = tmem + 8,
+                            total = hdr + sizeof(ScratchHdr);
 };
 constexpr uint32_t kFwdCols = 256;
 
@@ -354,6 +353,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
   float *ypart = reinterpret_cast<float *>(sm + FwdSmem::ypart);
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + FwdSmem::bar);
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + FwdSmem::tmem);
+  ScratchHdr *hdr = reinterpret_cast<ScratchHdr *>(sm + FwdSmem::hdr);
   uint8_t *Z = sm + FwdSmem::z;
   const uint32_t warp = threadIdx.x >> 5, half = warp >> 2, row = threadIdx.x & 127u;
   const bool vec = ((uintptr_t)x & 15u) == 0;
@@ -361,6 +361,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
   load_x<kFwdThreads>(x, B, (uint64_t)blockIdx.x * kTileS, vec, xr);
   if (warp == 0) tmem_alloc(slot, kFwdCols);
   if (threadIdx.x == 0) {
+    *hdr = ScratchHdr{};
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -383,7 +384,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
       for (uint32_t k = 0; k < 4; ++k) mma_ss(tm + 128 * (k >> 1), dx + 2 * k, dw1 + 2 * k, id, k & 1u);
       tc_commit(bar);
     }
-    ok = tc_wait(bar, phase, waits);
+    ok = tc_wait(bar, phase, hdr, waits);
     phase ^= 1u;
     tc_after_sync();
     float2 v[2][16];   // 32 units of either half of z1
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
       Split32 z;
       z.make<true>(v[h]);
       if (h == 1) {   // the first half's products have read Z
-        ok = tc_wait(bar, phase, waits) && ok;
+        ok = tc_wait(bar, phase, hdr, waits) && ok;
         phase ^= 1u;
       }
       z.store(Z, kBlock, 4 * half, row);
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
       }
     }
     if (!ok) break;
-    ok = tc_wait(bar, phase, waits);
+    ok = tc_wait(bar, phase, hdr, waits);
     phase ^= 1u;
     tc_after_sync();
     store_x<kFwdThreads>(sm + FwdSmem::x, xr);
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
     if (half == 0 && s0 + row < B) y[s0 + row] = part + ypart[row] + V.b3;   // (ypart is written again two barriers later)
   }
   if (!ok) {
-    mbar_wait(bar, phase ^ 1u, &g_mlp_hdr);   // the products in flight
+    mbar_wait(bar, phase ^ 1u, hdr);   // the products in flight
     for (; s0 < B; s0 += (uint64_t)gridDim.x * kTileS)
       if (half == 0 && s0 + row < B) y[s0 + row] = __int_as_float(0x7fffffff);
   }
@@ -482,14 +483,14 @@ __global__ void __launch_bounds__(kFwdThreads, 2) mlp_forward_kernel(const uint1
 // and conversions of one tile, the loading of weights, and the fetching of
 // instructions that each block runs once (20 us here by ncu, 24 with 256
 // threads and twice the code, 43 before the tensor cores).  A training step
-// (two fills, this, Adam): 4096 samples 50.5 -> 29 us, 20,000 162 -> 48, 65,536
-// 417 -> 79.  Of that, the tests for infinities, NaN and waits that gave up are
-// 0.5 us, 1 to 2 and 2 to 4.
+// (two fills, this, Adam): 4096 samples 50.5 -> 28.7 us, 20,000 162 -> 49, 65,536
+// 417 -> 82.  Of that, the tests for infinities, NaN and waits that gave up are
+// nothing that shows, 2 and 2 to 3 us.
 constexpr uint32_t kTgB = 384, kTm = 448, kTgW1 = 448;
 struct GradSmem {
   static constexpr uint32_t w1 = 0, w2 = kBlock, x = 3 * kBlock, e = 4 * kBlock, mask = 5 * kBlock, r = 7 * kBlock,
-                            vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * 4 * kTileS, tmem = bar + 16,
-                            bad = tmem + 16, bad_dy = bad + 16,
+                            vec = 13 * kBlock, part = vec + sizeof(MlpVectors), bar = part + 4 * 4 * kTileS, tmem = bar + 32,
+                            hdr = tmem + 16, bad = hdr + sizeof(ScratchHdr), bad_dy = bad + 16,
                             total = bad_dy + 4 * kTileS;
 };
 
@@ -513,8 +514,8 @@ __device__ __forceinline__ void add4(float *p, float a, float b, float c, float 
 // time, one for each 128 threads; `scratch`: shared memory.  The whole block
 // calls, and meets at a barrier before it leaves.  A gradient of 4096 samples
 // takes 35 us with one bad residual and 240 us with nothing but bad ones (19
-// without; 39 either way before the tensor cores), 1M samples 749 us and 12.5 ms
-// (747; 6.1 ms).
+// without; 39 either way before the tensor cores), 1M samples 748 us and 12.5 ms
+// (740; 6.1 ms).
 struct PlainRows {
   float z1[4][kH], d2[4][kH], d1[4][kH], red[4][4];
   uint8_t row[kTileS];
@@ -604,8 +605,9 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   extern __shared__ __align__(1024) uint8_t sm[];
   MlpVectors &V = *reinterpret_cast<MlpVectors *>(sm + GradSmem::vec);
   float *part = reinterpret_cast<float *>(sm + GradSmem::part);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [2]
+  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GradSmem::bar);   // [3]
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + GradSmem::tmem);
+  ScratchHdr *hdr = reinterpret_cast<ScratchHdr *>(sm + GradSmem::hdr);
   uint8_t *R = sm + GradSmem::r, *E = sm + GradSmem::e, *mask = sm + GradSmem::mask;
   uint32_t *bad = reinterpret_cast<uint32_t *>(sm + GradSmem::bad);   // the tile's samples left to add_samples (bits)
   float *bad_dy = reinterpret_cast<float *>(sm + GradSmem::bad_dy);
@@ -615,8 +617,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   load_x<kGradThreads>(x, B, (uint64_t)blockIdx.x * kTileS, vec, xr);
   if (warp == 0) tmem_alloc(slot, kTmCols);
   if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+    *hdr = ScratchHdr{};
+    for (int k = 0; k < 3; ++k) mbar_init(&bar[k], 1);
     bad[0] = bad[1] = bad[2] = bad[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -635,7 +637,9 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
   constexpr uint32_t kPart = 2 * (kBlock >> 4);   // descriptor distance of two parts of R
   constexpr uint32_t kRows16 = 2048 >> 4;         // of 16 rows (MN-major: a step of K)
   uint32_t ph0 = 0, ph1 = 0, waits = 0;
-  bool ok = true;   // as in the forward kernel
+  // No warp of the block has given up (after the two barriers below that agree on
+  // it, before the tile's first and last additions).
+  bool ok = true;
   float lsum = 0.0f, gb3 = 0.0f;
   const float inv_b = 2.0f / (float)B;
   for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
@@ -644,7 +648,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       tc_commit(&bar[0]);
     }
     const float target = s0 + row < B ? t[s0 + row] : 0.0f;
-    ok = tc_wait(&bar[0], ph0, waits);
+    ok = tc_wait(&bar[0], ph0, hdr, waits);
     ph0 ^= 1u;
     tc_after_sync();
     float2 z1[16], v[16];
@@ -654,14 +658,13 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     store_split32<true>(R, quarter, row, z1);
     fence_proxy_async_smem();
     tc_before_sync();
-    ok = __syncthreads_and(ok && !inf) != 0;
-    if (!ok) break;
+    __syncthreads();
     if (threadIdx.x == 0) {
       tc_after_sync();
       issue_layer2(tm, dr, dw2);
       tc_commit(&bar[0]);
     }
-    ok = tc_wait(&bar[0], ph0, waits);
+    ok = tc_wait(&bar[0], ph0, hdr, waits) && ok;
     ph0 ^= 1u;
     tc_after_sync();
     // y, the mask, mask w3
@@ -684,8 +687,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     // y of the row: the quarters' sums
     part[quarter * kTileS + row] = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
     tc_before_sync();
-    ok = __syncthreads_and(ok) != 0;   // (a2 has been read by all: its columns are free)
-    if (!ok) break;
+    __syncthreads();   // (a2 has been read by all: its columns are free)
     tc_after_sync();
     tmem_st16(lanes + kTm + 16 * quarter, mw);
     // (every quarter computes dy for itself; rows past the batch: 0, they add nothing)
@@ -716,7 +718,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(hi << 16, mid | lo << 16, 0, 0);
     }
     fence_proxy_async_smem();
-    ok = tc_wait(&bar[0], ph0, waits);
+    ok = tc_wait(&bar[0], ph0, hdr, waits) && ok;
     ph0 ^= 1u;
     tc_after_sync();
     load_sum32(mine, v);
@@ -727,10 +729,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     for (int k = 0; k < 16; ++k) odd = __ffma2_rn(z1[k], make_float2(0.0f, 0.0f), odd);
     const bool left_out = !(odd.x + odd.y == 0.0f);
     tc_before_sync();
-    if (__syncthreads_or(left_out || !ok)) {
-      ok = __syncthreads_and(ok) != 0;
-      if (!ok) break;
-      // those samples' operands become 0; add_samples makes up for them below
+    if (__syncthreads_or(left_out)) {   // those samples' operands become 0; add_samples makes up for them below
       if (left_out) atomicOr(&bad[row >> 5], 1u << (row & 31u));
       if (quarter == 0) bad_dy[row] = dy;
       __syncthreads();
@@ -754,14 +753,14 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       tc_commit(&bar[1]);
     }
     load_x<kGradThreads>(x, B, s0 + (uint64_t)gridDim.x * kTileS, vec, xr);
-    ok = tc_wait(&bar[1], ph1, waits);   // R and E are free
+    ok = tc_wait(&bar[1], ph1, hdr, waits) && ok;   // R and E are free
     ph1 ^= 1u;
     tc_after_sync();
     store_split32<false>(R, quarter, row, z1);
     if (quarter == 0) *reinterpret_cast<uint4 *>(chunk(E, row, 0)) = make_uint4(0x3f80u, 0, 0, 0);
     fence_proxy_async_smem();
     tc_before_sync();
-    ok = __syncthreads_and(ok) != 0;
+    ok = __syncthreads_and(ok && !inf) != 0;
     if (!ok) break;
     if (threadIdx.x == 0) {
       tc_after_sync();
@@ -803,7 +802,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
       if (any == 0.0f) dot = make_float2(0.0f, 0.0f);
     }
     part[quarter * kTileS + row] = dot.x + dot.y;   // (dy's sums have been read)
-    ok = tc_wait(&bar[0], ph0, waits);
+    ok = tc_wait(&bar[0], ph0, hdr, waits);
     ph0 ^= 1u;
     tc_after_sync();
     ok = __syncthreads_and(ok) != 0;
@@ -838,9 +837,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(const uint16_
     tc_after_sync();
   }
   if (!ok) {
-    mbar_wait(&bar[0], ph0 ^ 1u, &g_mlp_hdr);   // the products in flight
-    mbar_wait(&bar[1], ph1 ^ 1u, &g_mlp_hdr);
+    if (threadIdx.x == 0) tc_commit(&bar[2]);
+    mbar_wait(&bar[2], 0, hdr);   // the products in flight
     if (__syncthreads_or(inf)) {   // an infinity in W2 (the first tile has ended here): sample by sample
+      lsum = gb3 = 0.0f;
 #pragma unroll 1
       for (uint64_t s0 = (uint64_t)blockIdx.x * kTileS; s0 < B; s0 += (uint64_t)gridDim.x * kTileS) {
         const uint64_t left = B - s0;   // rows of the tile
